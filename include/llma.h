@@ -236,6 +236,11 @@ int llma_debug_timeline(llma_engine *e, int32_t clear, unsigned long long *out);
  * (1, 2 or 4; chosen at llma_create from max_batch, max_seq and the head count alone).  Errors: NULL. */
 int llma_debug_attention_tiles(llma_engine *e);
 
+/* Inspection: activation rows per tile of a prompt projection (0 QKV, 1 output, 2 gate/up, 3 down) in a pass of n_rows
+ * positions (64, 96 or 128; results do not depend on it), or a negative status.  Errors: NULL, ARG (which, n_rows < 1),
+ * STATE (an engine on the CUDA-core path). */
+int llma_debug_prompt_row_tile(llma_engine *e, int32_t which, int32_t n_rows);
+
 /* Rows the engine's activation buffers hold (the leading dimension of llma_debug_buffer), or a negative
  * status. */
 int llma_row_capacity(llma_engine *e);

@@ -148,6 +148,16 @@ extern "C" int llma_debug_timeline(llma_engine* e, int32_t clear, unsigned long 
     return LLMA_OK;
 }
 
+extern "C" int llma_debug_prompt_row_tile(llma_engine* e, int32_t which, int32_t n_rows) {
+    if (!e) return LLMA_ERR_NULL;
+    if (which < 0 || which > 3 || n_rows < 1) return LLMA_ERR_ARG;
+    if (e->gemm_impl != LLMA_GEMM_TCGEN05) return LLMA_ERR_STATE;
+    const ModelDims& d = e->dims;
+    const int tiles[4] = {3 * d.hd_total / 128, d.d_model / 128, d.d_ffn / 64, d.d_model / 128};
+    const int k_in[4] = {d.d_model, d.hd_total, d.d_model, d.d_ffn};
+    return prompt_row_tile(n_rows, (tiles[which] + 1) / 2, k_in[which] / 64, e->prompt_pairs);
+}
+
 extern "C" int llma_debug_attention_tiles(llma_engine* e) {
     if (!e) return LLMA_ERR_NULL;
     return e->attn_tiles;

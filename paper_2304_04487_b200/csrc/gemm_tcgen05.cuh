@@ -10,11 +10,12 @@
 // activation rows are its N operand, so every weight byte crosses HBM exactly once per
 // step however many rows are verified.  Work is the flat list of (tile, 64-wide k-chunk)
 // pairs, cut into equal contiguous ranges, one per CTA; partial tiles are summed in a fixed
-// order that depends on the matrix shape and grid only -- never on the rows in use.
+// order that depends on the matrix shape and grid only -- never on the rows in use.  (Prompt passes cut k into parts whose
+// length depends on k only, to the same end.)
 //
 // gemm_ws_kernel<NR> serves engines of at most 32 decoding rows (NR = 16 or 32 fixed per engine; activation tiles copied by
 // loader warps), gemm_wide_kernel up to 256 (activation tiles by TMA, MMA N = the rows in use rounded up, epilogue in
-// blocks of 32 rows), gemm_prompt_kernel the passes of a prompt (tiles of 256 features x N rows per CTA pair).
+// blocks of 32 rows), gemm_prompt_kernel the passes of a prompt (tiles of 256 features x 64 to 128 rows per CTA pair).
 #pragma once
 #include <cuda.h>
 
@@ -154,6 +155,7 @@ void launch_gemm_wide(cudaStream_t st, int grid, bool pdl, const GemmArgs& args,
 // Prompt passes of many rows (gemm_prompt.cu): kGemmQKV, kGemmResid and kGemmSwiGLU over n_rows rows.  a0..a2 as for
 // gemm_wide_kernel; act is the split activation buffer [2 rc][k_in].  `pairs` = CTA pairs that run at once.
 cudaError_t init_gemm_prompt(int* pairs);
+int prompt_row_tile(int n_rows, int feat_tiles, int chunks, int pairs);  // rows per tile that a launch takes
 int launch_gemm_prompt(cudaStream_t st, const GemmArgs& args, int n_rows, int pairs, const CUtensorMap& a0, const CUtensorMap& a1,
                        const CUtensorMap& a2);
 

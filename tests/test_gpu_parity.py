@@ -6,7 +6,7 @@ from oracle import decoding as D
 from oracle import model as OM
 from workloads import SHAPES, ModelShape, build_reference, make_prompt, make_weights
 
-from parity import BF16_LOGIT_TOL, step_parity, step_parity_batch
+from parity import BF16_LOGIT_TOL, gpu_kv_rows, step_parity, step_parity_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -506,3 +506,58 @@ def test_long_prompt_passes(d, heads, hd, ffn, P):
     (b,), _ = eng.llma_generate(N, 1, 0)
     assert a == b
     eng.llma_destroy()
+
+
+# ---- prompt projections: every tile width, row counts at the edges of tiles and passes ------------------------------
+def _kv_bits(eng, positions):
+    return [np.concatenate([r.view(np.uint32).ravel() for r in gpu_kv_rows(eng, 0, p)]) for p in positions]
+
+
+def test_prompt_rows_do_not_depend_on_the_pass():
+    """A position's K/V rows are the same bits whatever the length of its prompt, hence whatever the tile width, the rows
+    beside it in the tile and the pass it falls into; those of the longest prompt are compared with the oracle.  Width 1024:
+    two parts of 8 k-chunks, and nine in the down projection (66 chunks), the last of them ragged."""
+    shape = ModelShape("prompt-1024-4224", 2, 1024, 8, 128, 4224, 1000, "bf16")
+    w = _weights(shape, std=0.03)
+    longest = 2299                                                    # two passes
+    prompt = make_prompt(longest + 1, shape.vocab, seed=41)
+    eng = _engine(shape, w, max_seq=longest + 32, max_ref=8, max_k=1)
+    edges = sorted({0, 1, 1149, 1150, 1151, 1152, 1153, 2047, 2048, longest - 1} |
+                   {m * t + o for m in (32, 64, 96, 128) for t in (1, 2, 3, 5, 11) for o in (-1, 0, 1)})
+    eng.llma_prefill(0, prompt)
+    want = dict(zip(edges, _kv_bits(eng, edges)))
+    om = OM.OracleModel(shape, w, max_seq=longest + 32)
+    for p in range(longest):
+        om.forward(int(prompt[p]), p, want_logits=False, given_kv=gpu_kv_rows(eng, 0, p))
+    flips, violations, _, seen = om.code_stats
+    print(f"width 1024, {longest} positions: {flips:.0f} of {seen:.0f} codes differ")
+    assert violations == 0 and seen == 2 * 2 * 1024 * longest
+    used = set()
+    for rows in (1, 2, 31, 32, 33, 63, 64, 65, 95, 96, 97, 127, 128, 129, 191, 192, 193, 256, 257, 384, 385, 512, 640, 1100, 1535, 2047, 2048, 2049):
+        used |= {eng.llma_debug_prompt_row_tile(i, rows if rows <= 2048 else 1056) for i in range(4)}
+        eng.llma_prefill(0, prompt[:rows + 1])
+        at = [p for p in edges if p < rows] + [rows - 1]
+        for p, got in zip(at, _kv_bits(eng, at)):
+            if p in want:
+                assert np.array_equal(got, want[p]), (rows, p)
+    assert used == {64, 96, 128}
+    eng.llma_destroy()
+
+
+def test_prompt_codes_at_7b_widths():
+    """A prompt of 300 positions through the tile widths of long prompts (two rows of tiles at N = 128, four at N = 96), every
+    cached code against the oracle's."""
+    shape = SHAPES["llama7b-2layer"]
+    w = _weights(shape)
+    P, N, k = 301, 4, 4
+    prompt = make_prompt(P, shape.vocab, seed=42)
+    eng = _engine(shape, w, max_seq=P + N + 16, max_ref=64, max_k=k, keep_logits=True)
+    assert [eng.llma_debug_prompt_row_tile(i, P - 1) for i in range(4)] == [128, 96, 128, 96]
+    rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=P + N + 16), prompt, prompt[:40], None, 1, k, N, "bf16", prescribe_kv=True)
+    print(f"7B widths, 300 positions: {rep.code_flips} of {rep.codes_seen} codes differ, {rep.code_boundary_dist:.2f} of the tolerance")
+    assert rep.code_violations == 0 and rep.codes_seen >= 2 * 2 * 4096 * (P - 1)
+    # 0.45 % with hi and lo in accumulators of their own and k in parts, 0.58 % in passes of 128 rows through the kernel of
+    # batched decoding steps, 0.71 % with both terms in one accumulator over all of k (same inputs, every run the same)
+    assert rep.code_flips <= 0.005 * rep.codes_seen
+    eng.llma_destroy()
+    _cache.clear()
