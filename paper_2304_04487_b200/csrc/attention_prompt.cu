@@ -5,7 +5,10 @@
 // stages.  Nothing is combined across warps and nothing goes through global memory, where a pass of 128 rows in
 // attention_mma_kernel writes chunk partials for a merge kernel and reads every K/V tile once per 128 rows.
 // Bound by mma.sync: Q and P enter as hi + lo pairs, so a 16 x 64 tile costs 256 m16n8k16 MMAs at head_dim 128
-// against 64 ldmatrix.  The row tiles with the most positions start first.
+// against 64 ldmatrix.  The row tiles with the most positions start first.  A tile's P V has accumulators of its own and is added to
+// the running output rounded to nearest: mma.sync rounds its additions towards zero, and with the running output as accumulator
+// the cached codes of the next layer differ 6 % more often at 2299 positions (0.655 against 0.616 %).  Four 7B layers, 1535
+// positions: 3.04 -> 3.06 ms.
 #include <cuda.h>
 
 #include "attention_frag.cuh"
@@ -147,28 +150,41 @@ attention_prompt_kernel(const PromptAttnArgs a, const __grid_constant__ CUtensor
             }
             l_lo = __fmaf_rn(l_lo, f_lo, bl_lo); l_hi = __fmaf_rn(l_hi, f_hi, bl_hi);
             m_lo = n_lo; m_hi = n_hi;
-#pragma unroll
-            for (int i = 0; i < HD / 8; ++i) { o[i][0] *= f_lo; o[i][1] *= f_lo; o[i][2] *= f_hi; o[i][3] *= f_hi; }
             landed = mbar_wait(bar_v(st), par) && landed;
+            uint32_t ph[4][4], pl[4][4];
 #pragma unroll
             for (int kp = 0; kp < 4; ++kp) {
-                uint32_t ph[4], pl[4];
-                split_pack(sc[2 * kp][0], sc[2 * kp][1], ph[0], pl[0]);
-                split_pack(sc[2 * kp][2], sc[2 * kp][3], ph[1], pl[1]);
-                split_pack(sc[2 * kp + 1][0], sc[2 * kp + 1][1], ph[2], pl[2]);
-                split_pack(sc[2 * kp + 1][2], sc[2 * kp + 1][3], ph[3], pl[3]);
+                split_pack(sc[2 * kp][0], sc[2 * kp][1], ph[kp][0], pl[kp][0]);
+                split_pack(sc[2 * kp][2], sc[2 * kp][3], ph[kp][1], pl[kp][1]);
+                split_pack(sc[2 * kp + 1][0], sc[2 * kp + 1][1], ph[kp][2], pl[kp][2]);
+                split_pack(sc[2 * kp + 1][2], sc[2 * kp + 1][3], ph[kp][3], pl[kp][3]);
+            }
 #pragma unroll
-                for (int nn = 0; nn < HD / 16; ++nn) {
-                    const int row = kp * 16 + (mi & 1) * 8 + t8;
-                    const int col = nn * 16 + (mi >> 1) * 8;
-                    const uint32_t vaddr = tile_v(st) + (uint32_t)(col >> 6) * L::kBoxBytes + (uint32_t)row * 128 +
-                                           ((((uint32_t)(col & 63) >> 3) ^ ((uint32_t)row & 7u)) << 4);
-                    uint32_t b[4];
-                    ldsm_x4_trans(vaddr, b);
-                    mma_bf16(o[2 * nn], ph, b[0], b[1]);
-                    mma_bf16(o[2 * nn + 1], ph, b[2], b[3]);
-                    mma_bf16(o[2 * nn], pl, b[0], b[1]);
-                    mma_bf16(o[2 * nn + 1], pl, b[2], b[3]);
+            for (int n0 = 0; n0 < HD / 16; n0 += 2) {  // 32 columns of V: four accumulators for the tile, added to the running output
+                float pv[4][4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { pv[i][0] = pv[i][1] = pv[i][2] = pv[i][3] = 0.f; }
+#pragma unroll
+                for (int kp = 0; kp < 4; ++kp) {
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int row = kp * 16 + (mi & 1) * 8 + t8;
+                        const int col = (n0 + u) * 16 + (mi >> 1) * 8;
+                        const uint32_t vaddr = tile_v(st) + (uint32_t)(col >> 6) * L::kBoxBytes + (uint32_t)row * 128 +
+                                               ((((uint32_t)(col & 63) >> 3) ^ ((uint32_t)row & 7u)) << 4);
+                        uint32_t b[4];
+                        ldsm_x4_trans(vaddr, b);
+                        mma_bf16(pv[2 * u], ph[kp], b[0], b[1]);
+                        mma_bf16(pv[2 * u + 1], ph[kp], b[2], b[3]);
+                        mma_bf16(pv[2 * u], pl[kp], b[0], b[1]);
+                        mma_bf16(pv[2 * u + 1], pl[kp], b[2], b[3]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float (&a4)[4] = o[2 * n0 + i];
+                    a4[0] = __fmaf_rn(a4[0], f_lo, pv[i][0]); a4[1] = __fmaf_rn(a4[1], f_lo, pv[i][1]);
+                    a4[2] = __fmaf_rn(a4[2], f_hi, pv[i][2]); a4[3] = __fmaf_rn(a4[3], f_hi, pv[i][3]);
                 }
             }
             landed = __all_sync(0xffffffffu, landed);

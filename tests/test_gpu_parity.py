@@ -532,6 +532,9 @@ def test_prompt_rows_do_not_depend_on_the_pass():
     flips, violations, _, seen = om.code_stats
     print(f"width 1024, {longest} positions: {flips:.0f} of {seen:.0f} codes differ")
     assert violations == 0 and seen == 2 * 2 * 1024 * longest
+    # 0.319 %, as with attention in 32-position partials; 0.337 % when the running output is the tensor core's accumulator
+    # over all positions (same inputs, every run the same)
+    assert flips <= 0.0033 * seen
     used = set()
     for rows in (1, 2, 31, 32, 33, 63, 64, 65, 95, 96, 97, 127, 128, 129, 191, 192, 193, 256, 257, 384, 385, 512, 640, 1100, 1535, 2047, 2048, 2049):
         used |= {eng.llma_debug_prompt_row_tile(i, rows if rows <= 2048 else 1056) for i in range(4)}
