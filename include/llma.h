@@ -105,7 +105,8 @@ typedef struct {
 
 /*
  * Create an engine on the current CUDA device.  `cuda_stream` is a cudaStream_t (may be
- * NULL for the default stream); all work of the engine is issued on it.  Allocates the K/V
+ * NULL for the default stream, where steps are launched kernel by kernel because CUDA does not capture it;
+ * on any other stream they run as graphs, kept for the last 64 (n, k)); all work of the engine is issued on it.  Allocates the K/V
  * cache ([layer][seq][head][max_seq][head_dim], zero-filled), reference storage and
  * workspaces.  Supported: head_dim 64 or 128; d_model, n_heads*head_dim and d_ffn multiples
  * of 64; max_batch <= 256 and max_batch*(max_k+1) <= 256 rows per decoding step (the rows of a

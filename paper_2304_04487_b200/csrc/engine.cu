@@ -45,8 +45,8 @@ extern "C" const char* llma_strerror(int s) {
 
 static void free_engine(llma_engine* e) {
     if (!e) return;
-    for (auto& kv : e->step_graphs) cudaGraphExecDestroy(kv.second);
-    for (auto& kv : e->lone_graphs) if (kv.second) cudaGraphExecDestroy(kv.second);
+    for (auto* graphs : {&e->step_graphs, &e->lone_graphs})
+        for (auto& kv : *graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     cudaFree(e->seq_state); cudaFree(e->rows); cudaFree(e->ref);
     cudaFree(e->y); cudaFree(e->out_tok); cudaFree(e->x); cudaFree(e->qkv);
     cudaFree(e->logits); cudaFree(e->x_hat); cudaFree(e->attn); cudaFree(e->h);
@@ -92,6 +92,7 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     e->cfg = *cfg;
     e->device = dev;
     e->stream = (cudaStream_t)cuda_stream;
+    e->can_capture = e->stream != nullptr && e->stream != cudaStreamLegacy;
     e->bf16 = cfg->dtype == LLMA_DTYPE_BF16;
     const bool tc_ok = cfg->dtype == LLMA_DTYPE_BF16 && HD % 128 == 0 && cfg->d_model % 128 == 0;
     if (cfg->gemm_impl == LLMA_GEMM_TCGEN05 && !tc_ok) { delete e; return LLMA_ERR_CONFIG; }

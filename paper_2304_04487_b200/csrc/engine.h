@@ -96,8 +96,12 @@ struct llma_engine {
     float* h_logits = nullptr;              // kLogitStage floats (llma_debug_logits)
 
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    std::map<std::pair<int, int>, cudaGraphExec_t> step_graphs;  // keyed by (n, k): a step of llma_generate
-    std::map<std::pair<int, int>, cudaGraphExec_t> lone_graphs;  // keyed by (n, k): llma_step; null until the second use
+    // captured steps by (n, k): of llma_generate, and of llma_step (there null until the second use); at most kStepGraphs each
+    struct StepGraph { cudaGraphExec_t exec; uint64_t used; };
+    typedef std::map<std::pair<int, int>, StepGraph> StepGraphs;
+    StepGraphs step_graphs, lone_graphs;
+    uint64_t graph_clock = 0;
+    bool can_capture = true;     // false on the legacy default stream, which CUDA does not capture: steps are launched directly
     int64_t launches_per_step = 0;
     int64_t launch_counter = 0;  // kernels enqueued since it was last cleared
     bool last_step_valid = false;
@@ -110,6 +114,7 @@ struct llma_engine {
 
 namespace llma {
 constexpr int kPromptPassRows = 2048;  // most positions of a prompt pass (140 KB of buffers per position at the 7B widths)
+constexpr size_t kStepGraphs = 64;     // n is any positive number: the pair used longest ago makes room
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date
 void gemm_release_idle();  // gives back the scratch that llma_gemm_rows32_bf16 keeps between calls

@@ -395,29 +395,54 @@ static int check_nk(const llma_engine* e, int n, int k) {
     return LLMA_OK;
 }
 
+// The entry of (n, k), made (with no graph yet) if there is none
+static llma_engine::StepGraph& graph_entry(llma_engine* e, llma_engine::StepGraphs& graphs, int n, int k, bool* is_new) {
+    auto it = graphs.find({n, k});
+    *is_new = it == graphs.end();
+    if (*is_new) {
+        if (graphs.size() >= kStepGraphs) {  // nothing runs between calls: a graph can go at once
+            auto old = graphs.begin();
+            for (auto g = graphs.begin(); g != graphs.end(); ++g)
+                if (g->second.used < old->second.used) old = g;
+            if (old->second.exec) cudaGraphExecDestroy(old->second.exec);
+            graphs.erase(old);
+        }
+        it = graphs.insert({{n, k}, {nullptr, 0}}).first;
+    }
+    it->second.used = ++e->graph_clock;
+    return it->second;
+}
+
+template <typename Enqueue>
+static int capture(llma_engine* e, cudaGraphExec_t* out, Enqueue enqueue) {
+    cudaGraph_t g = nullptr;
+    const int64_t before = e->launch_counter;
+    CU_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
+    enqueue();
+    cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
+    e->launch_counter = before;
+    CU_TRY(ce);
+    ce = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    if (ce != cudaSuccess) *out = nullptr;
+    CU_TRY(ce);
+    return LLMA_OK;
+}
+
 static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
-    auto it = e->lone_graphs.find({n, k});
-    if (it == e->lone_graphs.end()) {  // a single step is cheaper launched kernel by kernel than captured
-        enqueue_tail(e, n, k, false, true);
-        enqueue_step_body(e, n, k, false);
+    auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
+    bool first = false;
+    llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k, &first);
+    if (first || !e->can_capture) {  // a single step is cheaper launched kernel by kernel than captured
+        enqueue();
         CU_TRY(cudaGetLastError());
-        e->lone_graphs[{n, k}] = nullptr;
         return LLMA_OK;
     }
-    if (!it->second) {
-        cudaGraph_t g = nullptr;
-        const int64_t before = e->launch_counter;
-        CU_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
-        enqueue_tail(e, n, k, false, true);
-        enqueue_step_body(e, n, k, false);
-        cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
-        e->launch_counter = before;
-        CU_TRY(ce);
-        ce = cudaGraphInstantiate(&it->second, g, 0);
-        cudaGraphDestroy(g);
-        if (ce != cudaSuccess) { it->second = nullptr; CU_TRY(ce); }
+    if (!g.exec) {
+        const int rc = capture(e, &g.exec, enqueue);
+        if (rc) return rc;
     }
-    CU_TRY(cudaGraphLaunch(it->second, e->stream));
+    CU_TRY(cudaGraphLaunch(g.exec, e->stream));
     return LLMA_OK;
 }
 
@@ -469,23 +494,36 @@ extern "C" int llma_step(llma_engine* e, int32_t n, int32_t k, int32_t* out_toke
     return LLMA_OK;
 }
 
+// A step of llma_generate as a graph, or no graph where the stream cannot be captured
 static int get_step_graph(llma_engine* e, int n, int k, cudaGraphExec_t* out) {
-    auto it = e->step_graphs.find({n, k});
-    if (it != e->step_graphs.end()) { *out = it->second; return LLMA_OK; }
-    cudaGraph_t g = nullptr;
-    const int64_t before = e->launch_counter;
-    CU_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_step_body(e, n, k, true);
-    cudaError_t ce = cudaStreamEndCapture(e->stream, &g);
-    e->launches_per_step = e->launch_counter - before;
-    e->launch_counter = before;
-    CU_TRY(ce);
-    cudaGraphExec_t ge = nullptr;
-    ce = cudaGraphInstantiate(&ge, g, 0);
-    cudaGraphDestroy(g);
-    CU_TRY(ce);
-    e->step_graphs[{n, k}] = ge;
-    *out = ge;
+    *out = nullptr;
+    if (!e->can_capture) return LLMA_OK;
+    bool is_new = false;
+    llma_engine::StepGraph& g = graph_entry(e, e->step_graphs, n, k, &is_new);
+    if (!g.exec) {
+        const int rc = capture(e, &g.exec, [&] {
+            const int64_t before = e->launch_counter;
+            enqueue_step_body(e, n, k, true);
+            e->launches_per_step = e->launch_counter - before;
+        });
+        if (rc) return rc;
+    }
+    *out = g.exec;
+    return LLMA_OK;
+}
+
+static int launch_steps(llma_engine* e, cudaGraphExec_t graph, int n, int k, int steps) {
+    for (int i = 0; i < steps; ++i) {
+        if (graph) {
+            CU_TRY(cudaGraphLaunch(graph, e->stream));
+        } else {
+            const int64_t before = e->launch_counter;
+            enqueue_step_body(e, n, k, true);
+            e->launches_per_step = e->launch_counter - before;
+            e->launch_counter = before;
+            CU_TRY(cudaGetLastError());
+        }
+    }
     return LLMA_OK;
 }
 
@@ -544,7 +582,8 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         }
         if (left <= 0) break;
         const int batch = (left + k) / (k + 1);
-        for (int i = 0; i < batch; ++i) CU_TRY(cudaGraphLaunch(graph, e->stream));
+        rc = launch_steps(e, graph, n, k, batch);
+        if (rc) return rc;
         launches += (int64_t)batch * e->launches_per_step;
         // the last look at the state brings the tokens too (a few kilobytes at most: it may be any look)
         const bool with_tokens = (size_t)(y_hi - y_lo) * d.max_batch <= 16384;
@@ -642,7 +681,8 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
     enqueue_tail(e, 1, 0, false, true);
     const int64_t tail_launches = e->launch_counter - before;
     e->launch_counter = before;
-    for (int i = 0; i < n_steps; ++i) CU_TRY(cudaGraphLaunch(graph, e->stream));
+    rc = launch_steps(e, graph, 1, 0, n_steps);
+    if (rc) return rc;
     CU_TRY(cudaEventRecord(e->ev1, e->stream));
     rc = pull_state(e);
     if (rc) return rc;

@@ -113,3 +113,53 @@ def test_microbench_mma_runs_and_rejects_bad_arguments():
     for bad in ((24, 1, 256, 0), (272, 1, 256, 0), (256, 3, 256, 0), (32, 1, 0, 0), (32, 1, 256, 5), (0, 1, 1, 0)):
         with pytest.raises(LlmaError):
             llma_microbench_mma(*bad)
+
+
+@pytest.mark.parametrize("name", ["tiny-fp32", "tiny-bf16"])
+def test_engine_on_the_default_stream(setup, name):
+    """cuda_stream = NULL: CUDA does not capture the legacy default stream, so every entry point has to do without graphs.
+    Same tokens as on a stream of its own, from the second step with the same (n, k) on too."""
+    import torch
+    Engine = setup[0]
+    shape = SHAPES[name]
+    w = make_weights(shape, seed=0)
+    prompt = make_prompt(20, shape.vocab, seed=1)
+    own = Engine(shape, w, max_seq=96, max_ref=64, max_k=4)
+    null = Engine(shape, w, max_seq=96, max_ref=64, max_k=4, stream=torch.cuda.default_stream())
+    assert null.stream.cuda_stream == 0
+    out = []
+    for eng in (own, null):
+        eng.llma_prefill(0, prompt)
+        (y,), st = eng.llma_generate(24, 1, 0)
+        eng.llma_set_reference(0, y)
+        steps = []
+        eng.llma_rewind(0)
+        for _ in range(5):
+            steps += eng.llma_step(1, 4)[0]
+        eng.llma_rewind(0)
+        (z,), sz = eng.llma_generate(24, 1, 4)
+        eng.llma_rewind(0)
+        sf = eng.llma_generate_forced(0, [(3, 2)] * 6, y[:12])
+        out.append((y, steps, z, st.steps, st.launches, sz.steps, sz.launches, sf.tokens, sf.launches))
+    assert out[0] == out[1]
+    assert out[0][2] == out[0][0] and out[0][1] == out[0][0][:len(out[0][1])]
+
+
+def test_more_step_shapes_than_graphs_are_kept(setup):
+    """Captured steps are kept for the last 64 (n, k); one that has made room for another is captured again."""
+    Engine, shape, w = setup
+    eng = Engine(shape, w, max_seq=64, max_ref=32, max_k=4)
+    eng.llma_prefill(0, make_prompt(20, shape.vocab, seed=1))
+    (y,), _ = eng.llma_generate(12, 1, 0)
+    eng.llma_set_reference(0, y)
+    for turn in range(3):
+        for n in range(1, 71):
+            eng.llma_rewind(0)
+            got = []
+            while len(got) < 6:
+                got += eng.llma_step(n, 4)[0]
+            assert got[:6] == y[:6], (turn, n)
+        for n in range(1, 71):
+            eng.llma_rewind(0)
+            (z,), _ = eng.llma_generate(6, n, 4)
+            assert z == y[:6], (turn, n)
