@@ -68,7 +68,9 @@ typedef struct {
     int32_t keep_logits;  /* 1: keep the last step's logits for llma_debug_logits */
 } llma_config;
 
-/* Device pointers.  Per-layer arrays are HOST arrays of n_layers device pointers. */
+/* Device pointers.  Per-layer arrays are HOST arrays of n_layers device pointers.  The projections and lm_head must lie on
+ * 16-byte boundaries (llma_create returns CONFIG otherwise); tok_emb and the norm gains need no more than their values'
+ * own alignment. */
 typedef struct {
     const void *tok_emb;           /* [vocab, d_model] */
     const void *lm_head;           /* [vocab, d_model] */
@@ -298,8 +300,8 @@ int llma_microbench_mma(int32_t n, int32_t regions, int32_t groups, int32_t comm
  * The engine's projection kernel on its own: out[r, n] = sum_k W[n, k] * a[r, k] for the 32
  * activation rows a step can hold (Eq. 3 evaluates k+1 <= 32 positions against every weight
  * matrix in one pass).  W: device, bf16, row-major [n_out, k_in]; a: device, bf16, row-major
- * [32, k_in]; out: device, fp32, row-major [32, n_out].  k_in must be a multiple of 64; W and a
- * 16-byte aligned.  Its split-k scratch (2.3 MB) is allocated on the first call and kept for the next ones, at
+ * [32, k_in]; out: device, fp32, row-major [32, n_out], overlapping neither.  k_in must be a multiple of 64; W on a
+ * 16-byte boundary (ARG otherwise), and a too for full speed.  Its split-k scratch (2.3 MB) is allocated on the first call and kept for the next ones, at
  * most four such blocks per device; they are given back when an engine is destroyed on that device.  Any number of
  * threads may call at once, each call with a block of its own; synchronous.  Errors: NULL, ARG, CONFIG (not an sm_100 device), CUDA, DEVICE_TIMEOUT.
  */

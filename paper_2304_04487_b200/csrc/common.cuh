@@ -82,6 +82,13 @@ template <typename T> __device__ __forceinline__ T from_f32(float v);
 template <> __device__ __forceinline__ float from_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// Four consecutive values of a vector that belongs to the caller (norm gains, embedding rows), read one by one: its alignment is
+// that of an element.
+__device__ __forceinline__ float4 load4_each(const float* p) { return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3)); }
+__device__ __forceinline__ float4 load4_each(const __nv_bfloat16* p) {
+    return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]), __bfloat162float(p[3]));
+}
+
 // Activations that feed a projection are kept in one of two layouts (rc = the engine's row capacity):
 //   kActF32    fp32 [rc][K]                         (CUDA-core GEMM)
 //   kActSplit  bf16 [2 rc][K]: row r holds hi = bf16(v), row rc + r holds lo = bf16(v - hi), so

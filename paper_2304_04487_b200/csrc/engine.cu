@@ -85,6 +85,16 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
             !w->w_gate[l] || !w->w_up[l] || !w->w_down[l])
             return LLMA_ERR_NULL;
 
+    // the kernels read weight rows in 16-byte pieces, gains and embeddings value by value
+    auto off = [](const void* p, size_t grid) { return reinterpret_cast<uintptr_t>(p) % grid != 0; };
+    const size_t value = cfg->dtype == LLMA_DTYPE_BF16 ? 2 : 4;
+    bool misaligned = off(w->tok_emb, value) || off(w->lm_head, 16) || off(w->final_norm, 4);
+    for (int l = 0; l < L; ++l) {
+        misaligned = misaligned || off(w->attn_norm[l], 4) || off(w->ffn_norm[l], 4);
+        for (const void* m : {w->wq[l], w->wk[l], w->wv[l], w->wo[l], w->w_gate[l], w->w_up[l], w->w_down[l]}) misaligned = misaligned || off(m, 16);
+    }
+    if (misaligned) return LLMA_ERR_CONFIG;
+
     int dev = 0;
     CU_TRY(cudaGetDevice(&dev));
     llma_engine* e = new (std::nothrow) llma_engine();

@@ -71,10 +71,11 @@ int gemm_device(int* dev_out, int* sms) {
     return LLMA_OK;
 }
 
-// TMA descriptor and one launch; `a` is the caller's [32][k_in].
+// TMA descriptor and one launch; `a` is the caller's [32][k_in].  A W off the 16-byte grid has no descriptor.
 int gemm_rows32_launch(const void* W, const void* a, float* out, int32_t n_out, int32_t k_in, float* ws,
                        int32_t* dev_err, int grid, cudaStream_t st) {
     CUtensorMap ma;
+    if (reinterpret_cast<uintptr_t>(a) % sizeof(__nv_bfloat16) || reinterpret_cast<uintptr_t>(out) % sizeof(float)) return LLMA_ERR_ARG;
     if (make_tensor_map_bf16_chunks(&ma, W, (uint64_t)n_out, (uint64_t)k_in, 128) != 0) return LLMA_ERR_ARG;
     GemmArgs g;
     std::memset(&g, 0, sizeof(g));

@@ -254,7 +254,7 @@ __device__ __forceinline__ void block_resid(const GemmArgs& g, int tile, int war
     const bool two = nj > 16;
     float4 v[8];
     each_row(two, [&](int u) { v[u] = __ldcg(reinterpret_cast<const float4*>(x + (int64_t)min(warp + 4 * u, nj - 1) * g.ld)); });
-    const float4 gn = __ldg(reinterpret_cast<const float4*>(g.gain_next + col));
+    const float4 gn = load4_each(g.gain_next + col);
     sync();
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(g.xs_out) + (int64_t)jb * g.n_out + col;
     const int64_t lo_term = (int64_t)g.rc * g.n_out;

@@ -201,7 +201,28 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
             // registers in between (a register copy of the next tile costs 64 of them, and with those the CTA
             // leaves no room on the SM for a CTA of the attention kernel).  A copy is issued as soon as its
             // stage is free and handed to the MMA warp when it has landed.
+            // The stand-alone product takes the caller's rows wherever they lie: rows off the 16-byte grid are fetched value by value.
+            const bool off_grid = MODE == kGemmStore && (reinterpret_cast<uintptr_t>(act) & 15) != 0;
+            auto issue_off_grid = [&](int q) {
+                const int it = q / KC;
+                int c = c_beg + it;
+                while (c >= C) c -= C;
+                const int chunk = c * KC + q % KC;
+                const uint32_t dst0 = sB + (uint32_t)(it % S) * kBBytes + (uint32_t)(q % KC) * kBTile;
+#pragma unroll 1
+                for (int unit = lane; unit < NR * 8; unit += 32) {
+                    const int r = unit >> 3, j = unit & 7;
+                    uint32_t v[4] = {0u, 0u, 0u, 0u};
+                    if (chunk < g.chunks) {
+                        const unsigned short* p = reinterpret_cast<const unsigned short*>(act + r * ld_bytes + (int64_t)chunk * 128 + j * 16);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i] = (uint32_t)__ldcg(p + 2 * i) | ((uint32_t)__ldcg(p + 2 * i + 1) << 16);
+                    }
+                    st_shared_v4(dst0 + (uint32_t)r * 128 + (uint32_t)((j ^ (r & 7)) << 4), make_uint4(v[0], v[1], v[2], v[3]));
+                }
+            };
             auto issue = [&](int q, int row_limit) {
+                if (off_grid) { issue_off_grid(q); return; }
                 const int it = q / KC;
                 int c = c_beg + it;
                 while (c >= C) c -= C;

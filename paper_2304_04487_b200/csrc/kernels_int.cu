@@ -362,10 +362,7 @@ __global__ void __launch_bounds__(128) embed_prompt_kernel(int d, int rc, const 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = warp; t < d / 128; t += 4) {  // d is a multiple of 128 on the tensor-core path
         const int col = t * 128 + lane * 4;
-        const uint2 e = __ldg(reinterpret_cast<const uint2*>(er + col));
-        const float4 gn = __ldg(reinterpret_cast<const float4*>(gain + col));
-        const float4 v = make_float4(__uint_as_float(e.x << 16), __uint_as_float(e.x & 0xffff0000u), __uint_as_float(e.y << 16),
-                                     __uint_as_float(e.y & 0xffff0000u));
+        const float4 v = load4_each(er + col), gn = load4_each(gain + col);
         *reinterpret_cast<float4*>(x + (int64_t)r * d + col) = v;
         store_act(xs, kActSplit, rc, r, col, d, v.x * gn.x);
         store_act(xs, kActSplit, rc, r, col + 1, d, v.y * gn.y);

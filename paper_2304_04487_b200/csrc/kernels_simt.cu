@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) rowgemm_kernel(const RowGemm g
 #pragma unroll 1
             for (int k = k0 + 4 * tid; k < k1; k += 4 * kWarps * 32) {
                 float4 gn = make_float4(1.f, 1.f, 1.f, 1.f);
-                if (kNorm && kStore) gn = __ldg(reinterpret_cast<const float4*>(g.gain + k));
+                if (kNorm && kStore) gn = load4_each(g.gain + k);
 #pragma unroll
                 for (int q = 0; q < kRB; q += 4) {  // four rows' loads in flight
                     if (q < nr) {

@@ -163,3 +163,63 @@ def test_more_step_shapes_than_graphs_are_kept(setup):
             eng.llma_rewind(0)
             (z,), _ = eng.llma_generate(6, n, 4)
             assert z == y[:6], (turn, n)
+
+
+class _OnDevice:
+    """Device tensors in the form in which one engine lends its weights to another."""
+
+    def __init__(self, dev):
+        self._dev = dev
+
+
+def _shifted(t, values=1):
+    """The same values `values` elements past a 256-byte boundary."""
+    import torch
+    flat = torch.empty(t.numel() + values, dtype=t.dtype, device=t.device)
+    flat[values:] = t.flatten()
+    return flat[values:].view(t.shape)
+
+
+@pytest.mark.parametrize("name,B,k,P", [("tiny-fp32", 1, 4, 40),      # CUDA cores
+                                        ("small-bf16", 1, 4, 200),    # prompt kernels, up to 16 rows
+                                        ("small-bf16", 5, 7, 100)])   # 33 to 256 rows
+def test_gains_and_embeddings_need_no_alignment(name, B, k, P):
+    """Norm gains and the embedding table may be views into larger buffers at any element: same bits as on a boundary."""
+    from paper_2304_04487_b200 import Engine
+    shape = SHAPES[name]
+    w = make_weights(shape, seed=0)
+    rng = np.random.default_rng(5)
+    for n in w:
+        if w[n].ndim == 1:
+            w[n] = rng.uniform(0.5, 1.5, w[n].shape).astype(np.float32)   # gains that differ from one another
+    a = Engine(shape, w, max_seq=P + 40, max_ref=32, max_k=k, max_batch=B, keep_logits=True)
+    dev = {n: _shifted(t) if t.ndim == 1 or n == "tok_emb" else t for n, t in a._dev.items()}
+    assert all(dev[n].data_ptr() % 16 for n in dev if dev[n].ndim == 1 or n == "tok_emb")
+    b = Engine(shape, None, max_seq=P + 40, max_ref=32, max_k=k, max_batch=B, keep_logits=True, share_weights_with=_OnDevice(dev))
+    out = []
+    for eng in (a, b):
+        for s in range(B):
+            eng.llma_prefill(s, make_prompt(P + s, shape.vocab, seed=s))
+            eng.llma_set_reference(s, make_prompt(P + s, shape.vocab, seed=s)[:32])
+        rows = []
+        for _ in range(4):
+            toks = eng.llma_step(1, k)
+            logits = eng.llma_debug_logits()
+            rows.append((toks, [logits[s * (k + 1):s * (k + 1) + i.k_eff + 1].copy() for s, i in enumerate(eng.llma_last_step_info())]))
+        out.append(rows)
+    for (ta, la), (tb, lb) in zip(*out):
+        assert ta == tb
+        assert all(np.array_equal(x, y) for x, y in zip(la, lb))
+
+
+@pytest.mark.parametrize("name", ["tiny-fp32", "tiny-bf16"])
+def test_misaligned_matrices_are_rejected(name):
+    from paper_2304_04487_b200 import Engine, LlmaError
+    shape = SHAPES[name]
+    a = Engine(shape, make_weights(shape, seed=0), max_seq=32, max_ref=8, max_k=2)
+    for n in ("wq.0", "wo.1", "w_up.0", "w_down.1", "lm_head"):
+        for impl in ((1,) if name == "tiny-fp32" else (1, 2)):
+            with pytest.raises(LlmaError) as ei:
+                Engine(shape, None, max_seq=32, max_ref=8, max_k=2, gemm_impl=impl,
+                       share_weights_with=_OnDevice({**a._dev, n: _shifted(a._dev[n])}))
+            assert ei.value.status == -2

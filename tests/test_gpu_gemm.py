@@ -82,3 +82,33 @@ def test_gemm_concurrent_calls(threads):
     for t in ts:
         t.join()
     assert not bad, bad
+
+
+@pytest.mark.parametrize("n_out,k_in", [(128, 64), (200, 192), (1000, 1024)])
+@pytest.mark.parametrize("shift", [1, 2, 4, 7])
+def test_rows_off_the_16_byte_grid(n_out, k_in, shift):
+    """The activation rows may lie anywhere (2-byte aligned), the result on any fp32: same bits as on a boundary."""
+    import torch
+    from paper_2304_04487_b200 import llma_gemm_rows32_bf16, llma_gemm_rows32_bf16_noalloc
+    W, a = (_to_dev(x) for x in _case(n_out, k_in, seed=9))
+    want = torch.empty((32, n_out), device="cuda")
+    llma_gemm_rows32_bf16(W, a, want)
+    flat = torch.empty(32 * k_in + shift, device="cuda", dtype=torch.bfloat16)
+    flat[shift:] = a.flatten()
+    rows = flat[shift:].view(32, k_in)
+    assert rows.data_ptr() % 16
+    for gemm in (llma_gemm_rows32_bf16, llma_gemm_rows32_bf16_noalloc):
+        res = torch.zeros(32 * n_out + 1, device="cuda")
+        gemm(W, rows, res[1:].view(32, n_out))
+        assert torch.equal(res[1:].view(32, n_out), want)
+
+
+def test_misaligned_operands_are_rejected():
+    import torch
+    from paper_2304_04487_b200 import lib
+    W, a = (_to_dev(x) for x in _case(128, 64, 0))
+    out = torch.empty(32 * 128 + 1, device="cuda")
+    for gemm in (lib().llma_gemm_rows32_bf16, lib().llma_gemm_rows32_bf16_noalloc):
+        assert gemm(W.data_ptr() + 2, a.data_ptr(), out.data_ptr(), 64, 64, None) == -9
+        assert gemm(W.data_ptr(), a.data_ptr() + 1, out.data_ptr(), 128, 64, None) == -9
+        assert gemm(W.data_ptr(), a.data_ptr(), out.data_ptr() + 2, 128, 64, None) == -9
