@@ -112,11 +112,8 @@ static void enqueue_forward_tc(llma_engine* e) {
     e->launch_counter += 1;
 }
 
-// most rows that one pass of a CUDA-core projection over its weights can meet (a multiple of 4, at most 16)
-static int row_bound(const llma_engine* e, bool decode) {
-    const int rows = decode ? e->dims.max_batch * e->dims.kp1 : e->prefill_rows;
-    return std::min(16, (rows + 3) / 4 * 4);
-}
+// most rows that a CUDA-core projection can meet in a decoding step or a prompt pass
+static int row_bound(const llma_engine* e, bool decode) { return decode ? e->dims.max_batch * e->dims.kp1 : e->prefill_rows; }
 
 static void enqueue_forward(llma_engine* e, bool lm_head) {
     if (e->gemm_impl == LLMA_GEMM_TCGEN05) { enqueue_forward_tc(e); return; }  // decoding steps only

@@ -67,11 +67,12 @@ struct RowGemm {
     float* part_max;        // kRowHead: [grid][row_cap]
     int32_t* part_idx;
     int32_t split_lg;       // set by launch_rowgemm: log2 of the warps that share a unit
+    int32_t pass_rows;      // ... and the rows that one pass over the weights takes
 };
 cudaError_t init_rowgemm(bool bf16);
-// row_bound: most rows of one pass (rows beyond 16 take further passes over the weights inside the launch)
+// row_bound: most rows of a step (more than a pass takes: further passes over the weights inside the launch)
 void launch_rowgemm(cudaStream_t st, bool bf16, RowGemm g, int row_bound, int num_sms);
-// CTAs of a launch (the number of partial maxima of kRowHead); row_bound a multiple of 4, at most 16
+// CTAs of a launch (the number of partial maxima of kRowHead)
 int rowgemm_grid(int n_units, int k_in, int row_bound, int num_sms);
 // causal attention of every used row over its sequence's cache rows [0, pos]; n_rows = the row slots of the pass
 void launch_attention_simt(cudaStream_t st, bool bf16, const ModelDims& dims, int layer, int n_rows,

@@ -25,7 +25,7 @@
 namespace llma {
 
 constexpr int kWarps = 8;        // warps per CTA
-constexpr int kRB = 16;          // activation rows per pass over the weights
+constexpr int kRB = 16;          // most activation rows per pass over the weights
 constexpr int kKC = 512;         // columns whose weights a warp holds at a time
 constexpr size_t kResidentBytes = 200 * 1024;  // activation rows that fit stay in shared memory whole
 
@@ -65,16 +65,23 @@ __device__ __forceinline__ float exchange32(float (&v)[32], int lane) {
     return v[0];
 }
 
-// RES: the activation rows fit shared memory whole (a kernel of its own, so that each carries one staging loop only: its code
-// is fetched anew by nearly every launch)
-template <typename T, int MODE, bool RES>
+// How the rows of a pass lie in shared memory; a kernel each, so that each carries one staging loop only (its code is fetched anew
+// by nearly every launch, and a pass length read from the arguments costs fp32 and bf16 widths of 192 to 512 another 1 to 2 %).
+enum Rows : int {
+    kChunked,  // a 512-wide chunk at a time, 16 rows a pass: not even four rows fit whole
+    kWhole,    // whole, 16 rows a pass
+    kFewer,    // whole, g.pass_rows (4, 8 or 12) a pass
+};
+template <typename T, int MODE, int ROWS>
 __global__ void __launch_bounds__(kWarps * 32, 2) rowgemm_kernel(const RowGemm g) {
     constexpr bool kNorm = MODE != kRowResid;  // the projections that read the residual stream
     constexpr int VN = Vec16<T>::N;
     constexpr int NV = kKC / (32 * VN);  // 16-byte pieces of a weight row per lane and chunk
     pdl_trigger();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr bool RES = ROWS != kChunked;
     const int K = g.k_in, KS = RES ? K : kKC;
+    const int pass = ROWS == kFewer ? g.pass_rows : kRB;
     extern __shared__ __align__(16) float sA[];  // [rows of a pass][KS]
     __shared__ float s_ss[kRB][kWarps];
     __shared__ float s_part[kWarps][32];
@@ -129,8 +136,8 @@ __global__ void __launch_bounds__(kWarps * 32, 2) rowgemm_kernel(const RowGemm g
     const int rows_used = __ldcg(&g.rows->rows_used);
 
 #pragma unroll 1
-    for (int r0 = 0; r0 < rows_used; r0 += kRB) {
-        const int nr = min(kRB, rows_used - r0);
+    for (int r0 = 0; r0 < rows_used; r0 += pass) {
+        const int nr = min(pass, rows_used - r0);
         if (r0 > 0) __syncthreads();
         // Rows r0 .. r0 + nr - 1, columns [k0, k1), into shared memory.  With kSquares every thread also adds up the squares of
         // its columns (the same columns of every row, so a row's sum has the same order whatever the number of rows).
@@ -216,9 +223,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2) rowgemm_kernel(const RowGemm g
                 uint4 w[2][NV];
 #pragma unroll
                 for (int i = 0; i < NV; ++i) { w[0][i] = w_next[0][i]; w[1][i] = w_next[1][i]; }
-                // the next turn's weights: of this unit, of the next one, or of the first one again for sixteen more rows
+                // the next turn's weights: of this unit, of the next one, or of the first one again for the next pass
                 const bool more = cc + 1 < n_turns, last = round + 1 == rounds;
-                if (more || !last || r0 + kRB < rows_used) load_weights(more ? round : (last ? 0 : round + 1), more ? c + split : part, w_next);
+                if (more || !last || r0 + pass < rows_used) load_weights(more ? round : (last ? 0 : round + 1), more ? c + split : part, w_next);
                 const int c0 = RES ? c * kKC : 0;
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
@@ -313,8 +320,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) rowgemm_kernel(const RowGemm g
 
 // ---- launchers -------------------------------------------------------------------------------
 template <typename T, int MODE>
-static cudaError_t opt_in() {  // the other instance stays within the default shared memory
-    return cudaFuncSetAttribute(rowgemm_kernel<T, MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentBytes);
+static cudaError_t opt_in() {  // the chunked instance stays within the default shared memory
+    const cudaError_t e = cudaFuncSetAttribute(rowgemm_kernel<T, MODE, kWhole>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentBytes);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(rowgemm_kernel<T, MODE, kFewer>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentBytes);
 }
 template <typename T>
 static cudaError_t opt_in_all() {
@@ -326,51 +335,67 @@ static cudaError_t opt_in_all() {
 }
 cudaError_t init_rowgemm(bool bf16) { return bf16 ? opt_in_all<__nv_bfloat16>() : opt_in_all<float>(); }
 
+// Rows per pass over the weights (a multiple of 4): 16, or fewer where 16 rows do not fit shared memory whole and fewer do; the
+// passes then share a step's rows evenly.  Fetching rows chunk by chunk, for every turn of the units and between two barriers, costs more
+// than reading the weights once more.  us per step, chunk by chunk -> whole in more passes (one warp per output before): two bf16
+// layers of width 4160, 16 rows 2831 -> 1283 (2157), 144 rows 24400 -> 10650 (17660); width 5184, 9 rows 3308 -> 1810 (2401); one of
+// width 8256, 5 rows 1767 -> 869 (964); two fp32 layers of width 4096, 16 rows 2562 -> 1420 (3314).
+static int pass_rows_of(int row_bound, int k_in) {
+    const int rows = (row_bound + 3) / 4 * 4;
+    const int most = (int)(kResidentBytes / (4 * sizeof(float) * k_in)) * 4;
+    if (most < 4 || most >= kRB) return rows < kRB ? rows : kRB;
+    const int passes = (rows + most - 1) / most;
+    return ((rows + passes - 1) / passes + 3) / 4 * 4;
+}
+static bool is_resident(int pass_rows, int k_in) { return (size_t)pass_rows * k_in * sizeof(float) <= kResidentBytes; }
+static int cta_cap(int k_in, int pass_rows, int num_sms) {  // CTAs that the GPU holds at once
+    return num_sms * (is_resident(2 * pass_rows, k_in) ? 2 : 1);
+}
 // Warps per unit: more than one where the units leave SMs without work and the columns make several chunks (output and down
 // projections of narrow decoders: 512 units of width 1024 are 64 CTAs).
-static int cta_cap(int k_in, int row_bound, int num_sms) {  // CTAs that the GPU holds at once
-    return num_sms * (2 * (size_t)row_bound * k_in * sizeof(float) <= kResidentBytes ? 2 : 1);
-}
-static int rowgemm_split(int n_units, int k_in, int row_bound, int num_sms) {
-    if ((size_t)row_bound * k_in * sizeof(float) > kResidentBytes) return 1;
-    const int cap = cta_cap(k_in, row_bound, num_sms), chunks = (k_in + kKC - 1) / kKC;
+static int rowgemm_split(int n_units, int k_in, int pass_rows, int num_sms) {
+    if (!is_resident(pass_rows, k_in)) return 1;
+    const int cap = cta_cap(k_in, pass_rows, num_sms), chunks = (k_in + kKC - 1) / kKC;
     int split = 1;
     while (split < 4 && 2 * split <= chunks && (n_units * 2 * split + kWarps - 1) / kWarps <= cap) split *= 2;
     return split;
 }
 // Beyond what the GPU holds at once the units are dealt in equal rounds.
 int rowgemm_grid(int n_units, int k_in, int row_bound, int num_sms) {
-    const int per_cta = kWarps / rowgemm_split(n_units, k_in, row_bound, num_sms), cap = cta_cap(k_in, row_bound, num_sms);
+    const int rows = pass_rows_of(row_bound, k_in);
+    const int per_cta = kWarps / rowgemm_split(n_units, k_in, rows, num_sms), cap = cta_cap(k_in, rows, num_sms);
     const int ctas = (n_units + per_cta - 1) / per_cta;
     const int rounds = (ctas + cap - 1) / cap;
     return (ctas + rounds - 1) / rounds;
 }
 
 template <typename T, int MODE>
-static void launch_mode(cudaStream_t st, int grid, size_t smem, bool resident, const RowGemm& g) {
-    if (resident) launch_pdl(st, true, dim3(grid), dim3(kWarps * 32), smem, rowgemm_kernel<T, MODE, true>, g);
-    else launch_pdl(st, true, dim3(grid), dim3(kWarps * 32), smem, rowgemm_kernel<T, MODE, false>, g);
+static void launch_mode(cudaStream_t st, int grid, size_t smem, Rows rows, const RowGemm& g) {
+    if (rows == kWhole) launch_pdl(st, true, dim3(grid), dim3(kWarps * 32), smem, rowgemm_kernel<T, MODE, kWhole>, g);
+    else if (rows == kFewer) launch_pdl(st, true, dim3(grid), dim3(kWarps * 32), smem, rowgemm_kernel<T, MODE, kFewer>, g);
+    else launch_pdl(st, true, dim3(grid), dim3(kWarps * 32), smem, rowgemm_kernel<T, MODE, kChunked>, g);
 }
 template <typename T>
-static void launch_typed(cudaStream_t st, int grid, size_t smem, bool resident, const RowGemm& g) {
+static void launch_typed(cudaStream_t st, int grid, size_t smem, Rows rows, const RowGemm& g) {
     switch (g.mode) {
-        case kRowQKV: launch_mode<T, kRowQKV>(st, grid, smem, resident, g); break;
-        case kRowResid: launch_mode<T, kRowResid>(st, grid, smem, resident, g); break;
-        case kRowSwiGLU: launch_mode<T, kRowSwiGLU>(st, grid, smem, resident, g); break;
-        default: launch_mode<T, kRowHead>(st, grid, smem, resident, g); break;
+        case kRowQKV: launch_mode<T, kRowQKV>(st, grid, smem, rows, g); break;
+        case kRowResid: launch_mode<T, kRowResid>(st, grid, smem, rows, g); break;
+        case kRowSwiGLU: launch_mode<T, kRowSwiGLU>(st, grid, smem, rows, g); break;
+        default: launch_mode<T, kRowHead>(st, grid, smem, rows, g); break;
     }
 }
 
 void launch_rowgemm(cudaStream_t st, bool bf16, RowGemm g, int row_bound, int num_sms) {
-    row_bound = row_bound < kRB ? (row_bound + 3) / 4 * 4 : kRB;
-    size_t smem = (size_t)row_bound * g.k_in * sizeof(float);
-    const bool resident = smem <= kResidentBytes;
-    if (!resident) smem = (size_t)row_bound * kKC * sizeof(float);
-    const int split = rowgemm_split(g.n_units, g.k_in, row_bound, num_sms);
+    g.pass_rows = pass_rows_of(row_bound, g.k_in);
+    const bool resident = is_resident(g.pass_rows, g.k_in);
+    const size_t smem = (size_t)g.pass_rows * (resident ? g.k_in : kKC) * sizeof(float);
+    const int split = rowgemm_split(g.n_units, g.k_in, g.pass_rows, num_sms);
     g.split_lg = split == 4 ? 2 : split - 1;
     const int grid = rowgemm_grid(g.n_units, g.k_in, row_bound, num_sms);
-    if (bf16) launch_typed<__nv_bfloat16>(st, grid, smem, resident, g);
-    else launch_typed<float>(st, grid, smem, resident, g);
+    // (a step of no more rows than a pass takes has one pass whatever its length)
+    const Rows rows = !resident ? kChunked : (g.pass_rows < kRB && row_bound > g.pass_rows ? kFewer : kWhole);
+    if (bf16) launch_typed<__nv_bfloat16>(st, grid, smem, rows, g);
+    else launch_typed<float>(st, grid, smem, rows, g);
 }
 
 }  // namespace llma

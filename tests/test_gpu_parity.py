@@ -564,3 +564,15 @@ def test_prompt_codes_at_7b_widths():
     assert rep.code_flips <= 0.005 * rep.codes_seen
     eng.llma_destroy()
     _cache.clear()
+
+
+# ---- CUDA-core projections whose rows do not fit shared memory sixteen at a time: 12, 8, 4 a pass, or chunk by chunk --------
+@pytest.mark.parametrize("d,ffn,dtype,k", [
+    (3264, 192, "fp32", 16),                     # width: 12 rows fit; 17 rows are passes of 12 and 5
+    (256, 3264, "bf16", 23),                     # down projection: two passes of 12
+    (256, 5184, "fp32", 8),                      # 8 fit: passes of 8 and 1
+    (256, 6464, "fp32", 4),                      # 4 fit: passes of 4 and 1
+    (256, 12800, "bf16", 6),                     # the most columns of which 4 rows fit
+    (64, 12864, "fp32", 18)])                    # beyond: chunk by chunk, 16 and 3 rows
+def test_cuda_core_rows_per_pass(d, ffn, dtype, k):
+    test_cuda_core_widths(d, 1, 64, ffn, 301, dtype, k, 1)
