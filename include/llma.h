@@ -302,8 +302,8 @@ int llma_microbench_mma(int32_t n, int32_t regions, int32_t groups, int32_t comm
  * matrix in one pass).  W: device, bf16, row-major [n_out, k_in]; a: device, bf16, row-major
  * [32, k_in]; out: device, fp32, row-major [32, n_out], overlapping neither.  k_in must be a multiple of 64; W on a
  * 16-byte boundary (ARG otherwise), and a too for full speed.  Its split-k scratch (2.3 MB) is allocated on the first call and kept for the next ones, at
- * most four such blocks per device; they are given back when an engine is destroyed on that device.  Any number of
- * threads may call at once, each call with a block of its own; synchronous.  Errors: NULL, ARG, CONFIG (not an sm_100 device), CUDA, DEVICE_TIMEOUT.
+ * most sixteen such blocks per device (one per concurrent call); they are given back with the last engine of that device.
+ * Any number of threads may call at once, each call with a block of its own; synchronous.  Errors: NULL, ARG, CONFIG (not an sm_100 device), CUDA, DEVICE_TIMEOUT.
  */
 int llma_gemm_rows32_bf16(const void *W, const void *a, float *out, int32_t n_out, int32_t k_in,
                           void *cuda_stream);

@@ -308,6 +308,7 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     CREATE_TRY(cudaEventCreate(&e->ev1));
     CREATE_TRY(cudaDeviceSynchronize());
 #undef CREATE_TRY
+    llma::gemm_count_engine(dev, 1);
     *out = e;
     return LLMA_OK;
 }
@@ -315,7 +316,8 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
 extern "C" int llma_destroy(llma_engine* e) {
     if (!e) return LLMA_OK;
     cudaStreamSynchronize(e->stream);
+    const int dev = e->device;
     free_engine(e);
-    gemm_release_idle();
+    llma::gemm_count_engine(dev, -1);
     return LLMA_OK;
 }

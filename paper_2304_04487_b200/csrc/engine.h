@@ -117,7 +117,7 @@ constexpr int kPromptPassRows = 2048;  // most positions of a prompt pass (140 K
 constexpr size_t kStepGraphs = 64;     // n is any positive number: the pair used longest ago makes room
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date
-void gemm_release_idle();  // gives back the scratch that llma_gemm_rows32_bf16 keeps between calls
+void gemm_count_engine(int dev, int by);  // the last engine of a device takes the scratch that llma_gemm_rows32_bf16 keeps with it
 void note_cuda_error(cudaError_t err);  // remembers the code for llma_last_cuda_error, clears the sticky flag
 }
 

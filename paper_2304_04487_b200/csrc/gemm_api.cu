@@ -16,7 +16,10 @@ using namespace llma;
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr size_t kMaxIdle = 4;  // blocks of 2.3 MB that a device keeps between calls; one is in use per concurrent call
+// Blocks of 2.3 MB that a device keeps between calls.  One is in use per concurrent call, and a call without one pays a cudaMalloc
+// and a cudaFree (milliseconds, and the device stops for them), so there are as many as callers a program may reasonably have
+// at once; 39 MB is the most that this can hold.
+constexpr size_t kMaxIdle = 16;
 
 // One call's scratch.  Between calls: every hand-over word all-ones, *err zero.
 struct Block {
@@ -29,6 +32,7 @@ struct Device {
     bool ready = false;
     int sms = 0;
     std::vector<Block> idle;
+    int engines = 0;  // alive on this device
 };
 Device g_dev[kMaxDevices];
 
@@ -88,16 +92,21 @@ int gemm_rows32_launch(const void* W, const void* a, float* out, int32_t n_out, 
     return LLMA_OK;
 }
 
-// Gives the idle scratch of the current device back (called when an engine goes; a later call allocates again).
-void gemm_release_idle() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
+// An engine has come (+1) or gone (-1).  With a device's last engine its idle scratch goes too (a later call allocates again).
+void gemm_count_engine(int dev, int by) {
+    if (dev < 0 || dev >= kMaxDevices) return;
     std::vector<Block> idle;
     {
         std::lock_guard<std::mutex> lock(g_dev[dev].mu);
-        idle.swap(g_dev[dev].idle);
+        g_dev[dev].engines += by;
+        if (by < 0 && g_dev[dev].engines == 0) idle.swap(g_dev[dev].idle);
     }
+    if (idle.empty()) return;
+    int current = 0;
+    cudaGetDevice(&current);
+    cudaSetDevice(dev);
     for (const Block& b : idle) free_block(b);
+    cudaSetDevice(current);
 }
 
 }  // namespace llma

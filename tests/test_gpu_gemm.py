@@ -54,7 +54,7 @@ def test_gemm_rejects_bad_arguments():
     assert L.llma_gemm_rows32_bf16(Wd.data_ptr(), ad.data_ptr(), out.data_ptr(), 0, 64, None) == -9
 
 
-@pytest.mark.parametrize("threads", [2, 6])                # fewer and more than the scratch blocks kept between calls
+@pytest.mark.parametrize("threads", [2, 6, 20])            # fewer and more than the scratch blocks kept between calls
 def test_gemm_concurrent_calls(threads):
     """Calls from several threads on streams of their own: each has scratch of its own, and it stays usable."""
     import threading
@@ -112,3 +112,35 @@ def test_misaligned_operands_are_rejected():
         assert gemm(W.data_ptr() + 2, a.data_ptr(), out.data_ptr(), 64, 64, None) == -9
         assert gemm(W.data_ptr(), a.data_ptr() + 1, out.data_ptr(), 128, 64, None) == -9
         assert gemm(W.data_ptr(), a.data_ptr(), out.data_ptr() + 2, 128, 64, None) == -9
+
+
+def test_scratch_outlives_all_but_the_last_engine():
+    """The product's scratch between calls: other engines' coming and going leaves it alone, the last one takes it along."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import torch
+from paper_2304_04487_b200 import Engine, llma_gemm_rows32_bf16
+from workloads import SHAPES, make_weights
+shape = SHAPES["tiny-fp32"]
+w = make_weights(shape, seed=0)
+free = lambda: (torch.cuda.synchronize(), torch.cuda.mem_get_info()[0])[1]
+W, a, out = torch.ones(512, 2816, device="cuda").bfloat16(), torch.ones(32, 2816, device="cuda").bfloat16(), torch.empty(32, 512, device="cuda")
+A = Engine(shape, w, max_seq=64, max_ref=8, max_k=1)
+B = Engine(shape, w, max_seq=64, max_ref=8, max_k=1)
+llma_gemm_rows32_bf16(W, a, out)
+A.llma_destroy()
+before = free()
+llma_gemm_rows32_bf16(W, a, out)
+assert free() == before, "scratch was allocated anew although an engine is left"
+C = Engine(shape, w, max_seq=64, max_ref=8, max_k=1)
+C.llma_destroy()
+B.llma_destroy()
+idle = free()
+llma_gemm_rows32_bf16(W, a, out)
+assert free() < idle, "scratch was kept past the last engine"
+assert float(out[0, 0]) == 2816.0
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
