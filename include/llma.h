@@ -134,7 +134,8 @@ int llma_prefill(llma_engine *e, int32_t seq, const int32_t *prompt, int32_t n_p
  * is the concatenation of n_docs documents; doc_offsets (host, n_docs+1 non-decreasing
  * values from 0 to n_tokens) delimits them, or NULL for a single document.  Neither the
  * matched n-gram nor the copied span crosses a document boundary.  n_tokens = 0 clears the
- * reference (plain greedy).  Copied to the device during the call.
+ * reference (plain greedy).  The arrays are copied before the call returns and may go then; the copy reaches the device
+ * in the order of the engine's stream, ahead of the next step, and a CUDA error on its way may surface in the next call.
  * Errors: NULL, REF_TOO_LONG, TOKEN_RANGE, CAPACITY, CUDA.
  */
 int llma_set_reference(llma_engine *e, int32_t seq, const int32_t *tokens, int32_t n_tokens,

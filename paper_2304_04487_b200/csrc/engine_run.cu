@@ -291,31 +291,24 @@ static int enqueue_prompt_pass(llma_engine* e, int seq, int p0, int n) {
     return bad ? LLMA_ERR_CONFIG : LLMA_OK;
 }
 
-extern "C" int llma_prefill(llma_engine* e, int32_t seq, const int32_t* prompt, int32_t n_prompt) {
-    if (!e || !prompt) return LLMA_ERR_NULL;
-    const ModelDims& d = e->dims;
-    if (seq < 0 || seq >= d.max_batch) return LLMA_ERR_CAPACITY;
-    if (n_prompt < 1) return LLMA_ERR_ARG;
-    if (n_prompt > d.max_seq) return LLMA_ERR_CAPACITY;
-    for (int i = 0; i < n_prompt; ++i)
-        if (prompt[i] < 0 || prompt[i] >= d.vocab) return LLMA_ERR_TOKEN_RANGE;
-    int rc = sync_state(e);
-    if (rc) return rc;
-    // push prompt[0 .. P-2] through the decoder
-    const int n_cache = n_prompt - 1;
-    if (e->gemm_impl == LLMA_GEMM_TCGEN05 && n_cache > 0) {  // passes of equal length
+// Tokens 0 .. n_cache - 1 of a prompt on their way through the decoder, into the K/V cache
+static int enqueue_prompt(llma_engine* e, int seq, const int32_t* prompt, int n_cache) {
+    if (e->gemm_impl == LLMA_GEMM_TCGEN05) {
+        if (n_cache == 0) return LLMA_OK;
+        // passes of equal length
         std::memcpy(e->h_y, prompt, (size_t)n_cache * sizeof(int32_t));
         CU_TRY(cudaMemcpyAsync(e->p_tok, e->h_y, (size_t)n_cache * sizeof(int32_t), cudaMemcpyHostToDevice, e->stream));
         const int passes = (n_cache + e->prompt_rc - 1) / e->prompt_rc;
         const int each = std::min(e->prompt_rc, ((n_cache + passes - 1) / passes + 31) / 32 * 32);
         for (int p0 = 0; p0 < n_cache; p0 += each) {
-            rc = enqueue_prompt_pass(e, seq, p0, std::min(each, n_cache - p0));
+            const int rc = enqueue_prompt_pass(e, seq, p0, std::min(each, n_cache - p0));
             if (rc) return rc;
         }
         CU_TRY(cudaGetLastError());
+        return LLMA_OK;
     }
     e->cur_rows = e->prefill_rows;
-    for (int p0 = 0; e->gemm_impl != LLMA_GEMM_TCGEN05 && p0 < n_cache; p0 += e->prefill_rows) {
+    for (int p0 = 0; p0 < n_cache; p0 += e->prefill_rows) {
         const int cnt = std::min(e->prefill_rows, n_cache - p0);
         RowDesc* R = e->h_rows;
         for (int r = 0; r < kRowCap; ++r) {
@@ -333,10 +326,29 @@ extern "C" int llma_prefill(llma_engine* e, int32_t seq, const int32_t* prompt, 
         CU_TRY(cudaGetLastError());
         CU_TRY(cudaStreamSynchronize(e->stream));  // h_rows is reused by the next chunk
     }
+    return LLMA_OK;
+}
+
+extern "C" int llma_prefill(llma_engine* e, int32_t seq, const int32_t* prompt, int32_t n_prompt) {
+    if (!e || !prompt) return LLMA_ERR_NULL;
+    const ModelDims& d = e->dims;
+    if (seq < 0 || seq >= d.max_batch) return LLMA_ERR_CAPACITY;
+    if (n_prompt < 1) return LLMA_ERR_ARG;
+    if (n_prompt > d.max_seq) return LLMA_ERR_CAPACITY;
+    for (int i = 0; i < n_prompt; ++i)
+        if (prompt[i] < 0 || prompt[i] >= d.vocab) return LLMA_ERR_TOKEN_RANGE;
+    int rc = sync_state(e);
+    if (rc) return rc;
+    // push prompt[0 .. P-2] through the decoder
+    rc = enqueue_prompt(e, seq, prompt, n_prompt - 1);
+    if (rc) {
+        cudaStreamSynchronize(e->stream);  // copies out of the staging memory may be under way: the next call writes to it
+        return rc;
+    }
     SeqState& S = e->h_state[seq];
     const int32_t keep_ref = S.ref_len;
     std::memset(&S, 0, sizeof(S));
-    S.active = 1; S.kv_len = n_cache; S.pending = prompt[n_prompt - 1]; S.ref_len = keep_ref;
+    S.active = 1; S.kv_len = n_prompt - 1; S.pending = prompt[n_prompt - 1]; S.ref_len = keep_ref;
     S.prompt_len = n_prompt; S.pos = -1; S.last_pos = -1; S.target_len = 0; S.done = 1;
     e->state_dirty = true;
     e->prompt_last[seq] = prompt[n_prompt - 1];
