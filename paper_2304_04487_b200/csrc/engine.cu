@@ -43,6 +43,12 @@ extern "C" const char* llma_strerror(int s) {
     }
 }
 
+static void free_prompt_buffers(llma_engine* e) {
+    for (void* b : {(void*)e->p_x, (void*)e->p_q, (void*)e->p_ss, e->p_x_hat, e->p_attn, e->p_h}) cudaFree(b);
+    e->p_x = e->p_q = e->p_ss = nullptr;
+    e->p_x_hat = e->p_attn = e->p_h = nullptr;
+}
+
 static void free_engine(llma_engine* e) {
     if (!e) return;
     for (auto* graphs : {&e->step_graphs, &e->lone_graphs})
@@ -53,7 +59,8 @@ static void free_engine(llma_engine* e) {
     cudaFree(e->rope_cos); cudaFree(e->rope_sin); cudaFree(e->kcache); cudaFree(e->vcache);
     cudaFree(e->attn_ws_o); cudaFree(e->attn_ws_ml); cudaFree(e->trace); cudaFree(e->target);
     cudaFree(e->gemm_ws); cudaFree(e->stamps); cudaFree(e->gemm_ws_wide); cudaFree(e->gemm_flags); cudaFree(e->part_max); cudaFree(e->part_idx); cudaFree(e->norm_ss);
-    cudaFree(e->p_tok); cudaFree(e->p_x); cudaFree(e->p_q); cudaFree(e->p_ss); cudaFree(e->p_x_hat); cudaFree(e->p_attn); cudaFree(e->p_h);
+    cudaFree(e->p_tok);
+    free_prompt_buffers(e);
     if (e->h_block) cudaFreeHost(e->h_block);
     for (int i = 0; i < 2; ++i)
         if (e->ref_ev[i]) cudaEventDestroy(e->ref_ev[i]);
@@ -61,6 +68,21 @@ static void free_engine(llma_engine* e) {
     if (e->ev0) cudaEventDestroy(e->ev0);
     if (e->ev1) cudaEventDestroy(e->ev1);
     delete e;
+}
+
+// The buffers of a prompt pass of prompt_rc positions, all of them or none
+static cudaError_t alloc_prompt_buffers(llma_engine* e) {
+    const ModelDims& d = e->dims;
+    const size_t rows = (size_t)e->prompt_rc;
+    cudaError_t r = dalloc(&e->p_x, rows * d.d_model, false);
+    if (r == cudaSuccess) r = dalloc(&e->p_q, rows * d.hd_total, false);
+    if (r == cudaSuccess) r = dalloc(&e->p_ss, rows * (d.d_model / 128), false);
+    // rows past a pass are multiplied too (their results go nowhere): zeroed, so that they stay finite
+    if (r == cudaSuccess) r = dalloc((char**)&e->p_x_hat, rows * d.d_model * 4);
+    if (r == cudaSuccess) r = dalloc((char**)&e->p_attn, rows * d.hd_total * 4);
+    if (r == cudaSuccess) r = dalloc((char**)&e->p_h, rows * d.d_ffn * 4);
+    if (r != cudaSuccess) free_prompt_buffers(e);
+    return r;
 }
 
 extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* cuda_stream, llma_engine** out) {
@@ -265,16 +287,16 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
         }
         CREATE_TRY(init_attention_mma());
         {
-            e->prompt_rc = std::min(kPromptPassRows, (d.max_seq - 1 + 31) / 32 * 32);
-            const size_t PC = (size_t)e->prompt_rc;
             CREATE_TRY(dalloc(&e->p_tok, (size_t)d.max_seq));
-            CREATE_TRY(dalloc(&e->p_x, PC * d.d_model, false));
-            CREATE_TRY(dalloc(&e->p_q, PC * HD, false));
-            CREATE_TRY(dalloc(&e->p_ss, PC * ((d.d_model + 127) / 128), false));
-            // rows past a pass are multiplied too (their results go nowhere): zeroed, so that they stay finite
-            CREATE_TRY(dalloc((char**)&e->p_x_hat, PC * d.d_model * 4));
-            CREATE_TRY(dalloc((char**)&e->p_attn, PC * HD * 4));
-            CREATE_TRY(dalloc((char**)&e->p_h, PC * d.d_ffn * 4));
+            // as many positions as a pass pays for, or fewer where memory is short (results do not depend on it)
+            e->prompt_rc = std::min(kPromptPassRows, (d.max_seq - 1 + 31) / 32 * 32);
+            cudaError_t pe = alloc_prompt_buffers(e);
+            while (pe == cudaErrorMemoryAllocation && e->prompt_rc > kPromptPassRowsMin) {
+                cudaGetLastError();
+                e->prompt_rc = std::max(kPromptPassRowsMin, e->prompt_rc / 64 * 32);
+                pe = alloc_prompt_buffers(e);
+            }
+            CREATE_TRY(pe);
             if (make_tensor_map_bf16(&e->map_kcache_64, e->kcache, kv_rows, d.head_dim, kPromptKV) ||
                 make_tensor_map_bf16(&e->map_vcache_64, e->vcache, kv_rows, d.head_dim, kPromptKV)) {
                 free_engine(e);

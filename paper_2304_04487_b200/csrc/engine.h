@@ -113,7 +113,8 @@ struct llma_engine {
 };
 
 namespace llma {
-constexpr int kPromptPassRows = 2048;  // most positions of a prompt pass (140 KB of buffers per position at the 7B widths)
+constexpr int kPromptPassRows = 2048;    // most positions of a prompt pass (110 KB of buffers per position at the 7B widths)
+constexpr int kPromptPassRowsMin = 128;  // ... and the fewest where memory is short
 constexpr size_t kStepGraphs = 64;     // n is any positive number: the pair used longest ago makes room
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date

@@ -223,3 +223,38 @@ def test_misaligned_matrices_are_rejected(name):
                 Engine(shape, None, max_seq=32, max_ref=8, max_k=2, gemm_impl=impl,
                        share_weights_with=_OnDevice({**a._dev, n: _shifted(a._dev[n])}))
             assert ei.value.status == -2
+
+
+def test_prompt_passes_shrink_where_memory_is_short():
+    """An engine whose full-sized prompt buffers do not fit takes smaller passes instead of failing: the same K/V rows.  (In a process
+    of its own, which takes all but part of the memory that the engine would like to have.)"""
+    import os
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch
+from paper_2304_04487_b200 import Engine
+from workloads import ModelShape, make_prompt, make_weights
+shape = ModelShape("wide-ffn", 1, 1024, 8, 128, 16384, 1000, "bf16")
+kw = dict(max_seq=2081, max_ref=8, max_k=1)
+a = Engine(shape, make_weights(shape, seed=0), **kw)
+prompt = make_prompt(2049, shape.vocab, seed=3)
+free = lambda: (torch.cuda.synchronize(), torch.cuda.mem_get_info()[0])[1]
+at = (0, 127, 128, 1023, 1024, 2047)
+def rows(eng):
+    eng.llma_prefill(0, prompt)
+    return [eng.llma_debug_kv_row(0, 0, p, which) for p in at for which in (0, 1)] + eng.llma_generate(4, 1, 0)[0]
+want = rows(a)
+before = free()
+b = Engine(shape, None, share_weights_with=a, **kw)
+size = before - free()
+b.llma_destroy()
+assert size > 168 << 20                       # 2048 positions of 82 KB, and the rest
+taken = torch.empty(free() - (size - (100 << 20)), dtype=torch.uint8, device="cuda")
+before = free()
+c = Engine(shape, None, share_weights_with=a, **kw)
+assert before - free() <= size - (80 << 20)
+assert all(np.array_equal(x, y) for x, y in zip(rows(c), want))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
