@@ -108,7 +108,8 @@ typedef struct {
 /*
  * Create an engine on the current CUDA device.  `cuda_stream` is a cudaStream_t (may be
  * NULL for the default stream, where steps are launched kernel by kernel because CUDA does not capture it;
- * on any other stream they run as graphs, kept for the last 64 (n, k)); all work of the engine is issued on it.  Allocates the K/V
+ * on any other stream they run as graphs, kept for the last 64 (n, k) and captured by llma_generate at once, by
+ * llma_step from the sixteenth use on); all work of the engine is issued on it.  Allocates the K/V
  * cache ([layer][seq][head][max_seq][head_dim], zero-filled), reference storage and
  * workspaces, among them, on the tensor-core path, 4 * (2 d_model + 2 n_heads*head_dim + d_ffn) bytes for each position of a
  * prompt pass (up to 2048 positions, 224 MB at the 7B widths; fewer positions, down to 128, where memory is short), and

@@ -96,8 +96,8 @@ struct llma_engine {
     float* h_logits = nullptr;              // kLogitStage floats (llma_debug_logits)
 
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // captured steps by (n, k): of llma_generate, and of llma_step (there null until the second use); at most kStepGraphs each
-    struct StepGraph { cudaGraphExec_t exec; uint64_t used; };
+    // captured steps by (n, k): of llma_generate, and of llma_step (there null until use kCaptureAt); at most kStepGraphs each
+    struct StepGraph { cudaGraphExec_t exec; uint64_t used; int uses; };
     typedef std::map<std::pair<int, int>, StepGraph> StepGraphs;
     StepGraphs step_graphs, lone_graphs;
     uint64_t graph_clock = 0;
@@ -116,6 +116,9 @@ namespace llma {
 constexpr int kPromptPassRows = 2048;    // most positions of a prompt pass (110 KB of buffers per position at the 7B widths)
 constexpr int kPromptPassRowsMin = 128;  // ... and the fewest where memory is short
 constexpr size_t kStepGraphs = 64;     // n is any positive number: the pair used longest ago makes room
+// llma_step launches kernel by kernel until an (n, k) has been used this often: capturing a step costs what a graph saves in 12 to
+// 23 of them (two layers of width 1024 115 against 10 us, three of width 512 170 against 8, the 7B shape 1400 against 60).
+constexpr int kCaptureAt = 16;
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date
 void gemm_count_engine(int dev, int by);  // the last engine of a device takes the scratch that llma_gemm_rows32_bf16 keeps with it

@@ -405,10 +405,9 @@ static int check_nk(const llma_engine* e, int n, int k) {
 }
 
 // The entry of (n, k), made (with no graph yet) if there is none
-static llma_engine::StepGraph& graph_entry(llma_engine* e, llma_engine::StepGraphs& graphs, int n, int k, bool* is_new) {
+static llma_engine::StepGraph& graph_entry(llma_engine* e, llma_engine::StepGraphs& graphs, int n, int k) {
     auto it = graphs.find({n, k});
-    *is_new = it == graphs.end();
-    if (*is_new) {
+    if (it == graphs.end()) {
         if (graphs.size() >= kStepGraphs) {  // nothing runs between calls: a graph can go at once
             auto old = graphs.begin();
             for (auto g = graphs.begin(); g != graphs.end(); ++g)
@@ -416,7 +415,7 @@ static llma_engine::StepGraph& graph_entry(llma_engine* e, llma_engine::StepGrap
             if (old->second.exec) cudaGraphExecDestroy(old->second.exec);
             graphs.erase(old);
         }
-        it = graphs.insert({{n, k}, {nullptr, 0}}).first;
+        it = graphs.insert({{n, k}, {nullptr, 0, 0}}).first;
     }
     it->second.used = ++e->graph_clock;
     return it->second;
@@ -440,9 +439,9 @@ static int capture(llma_engine* e, cudaGraphExec_t* out, Enqueue enqueue) {
 
 static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
     auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
-    bool first = false;
-    llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k, &first);
-    if (first || !e->can_capture) {  // a single step is cheaper launched kernel by kernel than captured
+    llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k);
+    if (!e->can_capture || g.uses + 1 < kCaptureAt) {
+        ++g.uses;
         enqueue();
         CU_TRY(cudaGetLastError());
         return LLMA_OK;
@@ -507,8 +506,7 @@ extern "C" int llma_step(llma_engine* e, int32_t n, int32_t k, int32_t* out_toke
 static int get_step_graph(llma_engine* e, int n, int k, cudaGraphExec_t* out) {
     *out = nullptr;
     if (!e->can_capture) return LLMA_OK;
-    bool is_new = false;
-    llma_engine::StepGraph& g = graph_entry(e, e->step_graphs, n, k, &is_new);
+    llma_engine::StepGraph& g = graph_entry(e, e->step_graphs, n, k);
     if (!g.exec) {
         const int rc = capture(e, &g.exec, [&] {
             const int64_t before = e->launch_counter;

@@ -118,7 +118,7 @@ def test_microbench_mma_runs_and_rejects_bad_arguments():
 @pytest.mark.parametrize("name", ["tiny-fp32", "tiny-bf16"])
 def test_engine_on_the_default_stream(setup, name):
     """cuda_stream = NULL: CUDA does not capture the legacy default stream, so every entry point has to do without graphs.
-    Same tokens as on a stream of its own, from the second step with the same (n, k) on too."""
+    Same tokens as on a stream of its own, whether a step is launched directly or replayed."""
     import torch
     Engine = setup[0]
     shape = SHAPES[name]
@@ -132,10 +132,12 @@ def test_engine_on_the_default_stream(setup, name):
         eng.llma_prefill(0, prompt)
         (y,), st = eng.llma_generate(24, 1, 0)
         eng.llma_set_reference(0, y)
-        steps = []
-        eng.llma_rewind(0)
-        for _ in range(5):
-            steps += eng.llma_step(1, 4)[0]
+        for _ in range(5):                     # 25 steps: launched directly, captured, replayed
+            steps = []
+            eng.llma_rewind(0)
+            for _ in range(5):
+                steps += eng.llma_step(1, 4)[0]
+            assert steps == y[:len(steps)]
         eng.llma_rewind(0)
         (z,), sz = eng.llma_generate(24, 1, 4)
         eng.llma_rewind(0)
