@@ -259,16 +259,16 @@ int llma_kv_len(llma_engine *e, int32_t seq);
 enum {
     LLMA_K_PLAN = 0,      /* trigger search + copy planning (the step-tail kernel launched for the plan alone) */
     LLMA_K_EMBED,         /* embedding gather */
-    LLMA_K_NORM,          /* RMSNorm */
+    LLMA_K_NORM,          /* unused: norms are folded into the projections */
     LLMA_K_GEMM_QKV,      /* QKV projection (tensor-core path: + rotary + K/V append) */
     LLMA_K_ATTN,          /* causal attention over the K/V cache */
     LLMA_K_GEMM_O,        /* output projection + residual */
     LLMA_K_GEMM_GATEUP,   /* gate/up projections (tensor-core path: + SiLU gating) */
     LLMA_K_GEMM_DOWN,     /* down projection + residual */
     LLMA_K_GEMM_LMHEAD,   /* LM head (tensor-core path: + per-tile argmax) */
-    LLMA_K_ARGMAX,        /* final per-row argmax (CUDA-core path; folded into ACCEPT on the tensor-core path) */
+    LLMA_K_ARGMAX,        /* unused: the final argmax is part of ACCEPT */
     LLMA_K_ACCEPT,        /* final argmax + acceptance + K/V commit (+ the next step's plan inside llma_generate) */
-    LLMA_K_EPILOGUE,      /* separate rotary / gating kernels of the SIMT path */
+    LLMA_K_EPILOGUE,      /* unused: rotary embedding and gating are part of the projections */
     LLMA_K_COUNT
 };
 

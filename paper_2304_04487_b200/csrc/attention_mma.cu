@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(128, 3) attention_mma_kernel(const AttnArgs a,
     const int kv_len = __ldcg(&a.seq_state[seq].kv_len);
     const bool early = c0 + kAttnChunk <= kv_len;
     if (threadIdx.x == 0) {
-        mbar_init(bar_u, 1); mbar_init(bar_v, 1); fence_mbar_init(); flag[0] = 0; flag[1] = 0;
+        mbar_init(bar_u, 1); mbar_init(bar_v, 1); fence_mbar_init(); flag[0] = 0;
         if (early) fetch_kv();
     }
     pdl_wait();  // row descriptors, q and the K/V rows of this step come from the kernels before
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(128, 3) attention_long_kernel(const AttnArgs a
     const int kv_len = __ldcg(&a.seq_state[seq].kv_len);
     const bool early = c0 + kAttnChunk <= kv_len;
     if (threadIdx.x == 0) {
-        mbar_init(bar_u, 1); mbar_init(bar_v, 1); fence_mbar_init(); flag[0] = 0; flag[1] = 0;
+        mbar_init(bar_u, 1); mbar_init(bar_v, 1); fence_mbar_init(); flag[0] = 0;
         if (early) { fetch_k(0); fetch_v(0); }
     }
     pdl_wait();
@@ -690,11 +690,9 @@ __global__ void __launch_bounds__(128) attention_merge_kernel(const AttnArgs a) 
     if (lane == 0) LLMA_STAMP_MINMAX(stp, 6);
 }
 
-constexpr size_t kAttnPad = 0;  // extra shared memory per CTA (a knob for the number of CTAs per SM)
-
 cudaError_t init_attention_mma() {
     cudaError_t e = cudaFuncSetAttribute(attention_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(AttnSmem<128>::kBytes + 1024 + kAttnPad));
+                                         (int)(AttnSmem<128>::kBytes + 1024));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attention_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(AttnSmem<64>::kBytes + 1024));
@@ -729,7 +727,7 @@ void launch_attention_mma(cudaStream_t st, const AttnArgs& a, const CUtensorMap&
         return;
     }
     if (a.dims.head_dim == 128) {
-        launch_pdl(st, true, grid, dim3(128), AttnSmem<128>::kBytes + 1024 + kAttnPad, attention_mma_kernel<128>, a, map_k, map_v);
+        launch_pdl(st, true, grid, dim3(128), AttnSmem<128>::kBytes + 1024, attention_mma_kernel<128>, a, map_k, map_v);
         launch_pdl(st, true, mgrid, dim3(128), msmem, attention_merge_kernel<128>, a);
     } else {
         launch_pdl(st, true, grid, dim3(128), AttnSmem<64>::kBytes + 1024, attention_mma_kernel<64>, a, map_k, map_v);

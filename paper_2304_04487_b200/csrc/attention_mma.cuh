@@ -18,7 +18,7 @@ struct AttnArgs {
     const SeqState* seq_state;  // decode steps: kv_len here is the length committed before this step
     int32_t n_rows;          // row slots of this pass (grid of the merge kernel)
     const float* qkv;        // [rows][3*H*hd] fp32, q already rotated
-    void* attn_out;          // ActLayout kActSplit [2 rc][H*hd]
+    void* attn_out;          // split bf16 [2 rc][H*hd]
     float* ws_o;             // chunk partials [head][chunk][rc][hd] fp32
     float* ws_ml;            // [head][chunk][rc][2] = (max, sum)
     unsigned long long* stamps;  // measurement builds: timeline block (see LLMA_STAMPS), else unused
@@ -35,7 +35,7 @@ struct PromptAttnArgs {
     int32_t layer, seq;
     int32_t pos0, n_rows;    // row r is position pos0 + r
     const float* q;          // [rows][H*hd] fp32, rotated
-    void* attn_out;          // ActLayout kActSplit [2 rc][H*hd]
+    void* attn_out;          // split bf16 [2 rc][H*hd]
     int32_t rc;
     int32_t* dev_err;
 };

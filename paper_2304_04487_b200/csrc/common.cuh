@@ -89,22 +89,14 @@ __device__ __forceinline__ float4 load4_each(const __nv_bfloat16* p) {
     return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]), __bfloat162float(p[3]));
 }
 
-// Activations that feed a projection are kept in one of two layouts (rc = the engine's row capacity):
-//   kActF32    fp32 [rc][K]                         (CUDA-core GEMM)
-//   kActSplit  bf16 [2 rc][K]: row r holds hi = bf16(v), row rc + r holds lo = bf16(v - hi), so
-//              hi + lo carries 16 mantissa bits through a bf16 tensor-core product (the two halves
-//              are summed in fp32)
-enum ActLayout : int32_t { kActF32 = 0, kActSplit = 1 };
-
-__device__ __forceinline__ void store_act(void* buf, int layout, int rc, int r, int64_t i, int64_t K, float v) {
-    if (layout == kActF32) {
-        reinterpret_cast<float*>(buf)[(int64_t)r * K + i] = v;
-    } else {
-        __nv_bfloat16* b = reinterpret_cast<__nv_bfloat16*>(buf);
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        b[(int64_t)r * K + i] = hi;
-        b[(int64_t)(rc + r) * K + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
+// Activations that feed a projection (rc = the engine's row capacity): fp32 [rc][K] for the CUDA-core kernels, split bf16 [2 rc][K] for
+// the tensor cores: row r holds hi = bf16(v), row rc + r holds lo = bf16(v - hi), so hi + lo carries 16 mantissa bits through a
+// bf16 product (the two halves are summed in fp32).
+__device__ __forceinline__ void store_split(void* buf, int rc, int r, int64_t i, int64_t K, float v) {
+    __nv_bfloat16* b = reinterpret_cast<__nv_bfloat16*>(buf);
+    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+    b[(int64_t)r * K + i] = hi;
+    b[(int64_t)(rc + r) * K + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
 // Every kernel of a decoding step is launched with programmatic stream serialization: it may

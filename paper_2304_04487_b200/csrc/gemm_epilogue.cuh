@@ -1,8 +1,7 @@
 // Epilogues of the weight-streaming GEMM: what happens to a finished 128 x 32 fp32 block.
 // Called by the 128 epilogue threads after the block has been staged in shared memory:
 // stage[f][j] is the result for output feature f of the tile (thread `row` staged its own
-// feature) and activation row jb + j, j < nj <= 32.  Engines of at most 32 rows have one
-// block per tile (jb = 0); the wide kernel walks a tile in blocks of 32 rows.
+// feature) and activation row j < nj <= 32 (gemm_ws_kernel: one block per tile).
 // red_f / red_i are [4][32] scratch for per-warp reductions.  With live = false nothing is stored to global memory
 // (the turn that only brings the code in).
 //
@@ -29,26 +28,23 @@ __device__ __forceinline__ float warp_sum(float v) {
 // x[r, n] += acc  (output projection and FFN down projection, residual stream in fp32).
 // When the next RMSNorm is folded in (g.xs_out): also xs = split(x * gain) and this tile's
 // per-row sums of squares, reduced over the 128 columns in an order fixed by the column index.
-// With kHavePre (jb = 0 only), xpre holds x[0..11, col] and the gain, read earlier by the caller.
-template <bool kHavePre>
-__device__ __forceinline__ void epilogue_resid(const GemmArgs& g, int tile, int row, int jb, int nj,
-                                               float (*stage)[33], float* red_f, const float (&xpre)[kXPre], bool live) {
+// xpre holds x[0..11, col] and the gain, read earlier by the caller.
+__device__ __forceinline__ void epilogue_resid(const GemmArgs& g, int tile, int row, int nj, float (*stage)[33],
+                                               const float (&xpre)[kXPre], bool live) {
     const int col = tile * 128 + row;
     const bool valid = col < g.n_out;
     const bool fold = g.xs_out != nullptr;
-    const float gain = kHavePre ? xpre[kXPre - 1] : ((fold && valid) ? __ldg(&g.gain_next[col]) : 0.f);
+    const float gain = xpre[kXPre - 1];
     const unsigned group = 0xffu << (row & 24);  // the eight lanes that share an activation row below
     // x is added into the staged tile with a few loads in flight; the per-row work is a rolled loop
-    if (kHavePre) {
 #pragma unroll
-        for (int u = 0; u < kXPre - 1; ++u)
-            if (u < nj) stage[row][u] += xpre[u];
-    }
-    for (int j0 = kHavePre ? kXPre - 1 : 0; j0 < nj; j0 += 8) {
+    for (int u = 0; u < kXPre - 1; ++u)
+        if (u < nj) stage[row][u] += xpre[u];
+    for (int j0 = kXPre - 1; j0 < nj; j0 += 8) {
         float xv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            xv[u] = (valid && j0 + u < nj) ? __ldcg(&g.out_f32[(int64_t)(jb + j0 + u) * g.ld + col]) : 0.f;
+            xv[u] = (valid && j0 + u < nj) ? __ldcg(&g.out_f32[(int64_t)(j0 + u) * g.ld + col]) : 0.f;
 #pragma unroll
         for (int u = 0; u < 8; ++u)
             if (j0 + u < nj) stage[row][j0 + u] += xv[u];
@@ -59,8 +55,8 @@ __device__ __forceinline__ void epilogue_resid(const GemmArgs& g, int tile, int 
 #pragma unroll 1
         for (int j = 0; j < nj; ++j) {
             const float xn = stage[row][j];
-            if (live) g.out_f32[(int64_t)(jb + j) * g.ld + col] = xn;
-            if (fold && live) store_act(g.xs_out, kActSplit, g.rc, jb + j, col, g.n_out, xn * gain);
+            if (live) g.out_f32[(int64_t)j * g.ld + col] = xn;
+            if (fold && live) store_split(g.xs_out, g.rc, j, col, g.n_out, xn * gain);
         }
     }
     if (!fold) return;
@@ -75,28 +71,25 @@ __device__ __forceinline__ void epilogue_resid(const GemmArgs& g, int tile, int 
         sq += __shfl_xor_sync(group, sq, 1);
         sq += __shfl_xor_sync(group, sq, 2);
         sq += __shfl_xor_sync(group, sq, 4);
-        if ((row & 7) == 0 && live) g.ss_out[(int64_t)tile * g.rc + jb + j] = sq;
+        if ((row & 7) == 0 && live) g.ss_out[(int64_t)tile * g.rc + j] = sq;
     }
     epi_sync();
 }
 
 // out[r, n] = acc
-__device__ __forceinline__ void epilogue_store(const GemmArgs& g, int tile, int row, int jb, int nj,
-                                               float (*stage)[33]) {
+__device__ __forceinline__ void epilogue_store(const GemmArgs& g, int tile, int row, int nj, float (*stage)[33]) {
     const int col = tile * 128 + row;
     if (col >= g.n_out) return;
 #pragma unroll 1
-    for (int j = 0; j < nj; ++j) g.out_f32[(int64_t)(jb + j) * g.ld + col] = stage[row][j];
+    for (int j = 0; j < nj; ++j) g.out_f32[(int64_t)j * g.ld + col] = stage[row][j];
 }
 
 // QKV: rotary embedding on q and k (pair (i, i + hd/2)), q to the fp32 qkv buffer, k and v
 // rows into the bf16 cache at (sequence, position) of every used row.
 //   row_pos[r] / row_seq[r]: position (-1: unused) and sequence slot of activation row r;
-//   rope_s: (cos, sin) of rows jb .. jb+31 staged in shared memory, [j][hd/2], or nullptr to read
-//   the tables in global memory.
-__device__ __forceinline__ void epilogue_qkv(const GemmArgs& g, int tile, int row, int jb, int nj,
-                                             float (*stage)[33], const int* row_pos, const int* row_seq,
-                                             const float2* rope_s, bool live) {
+//   rope_s: (cos, sin) of every row's position, staged in shared memory, [j][hd/2].
+__device__ __forceinline__ void epilogue_qkv(const GemmArgs& g, int tile, int row, int nj, float (*stage)[33], const int* row_pos,
+                                             const int* row_seq, const float2* rope_s, bool live) {
     const ModelDims& d = g.dims;
     const int mat = (tile >= g.tiles_per_map ? 1 : 0) + (tile >= 2 * g.tiles_per_map ? 1 : 0);
     const int col = (tile - mat * g.tiles_per_map) * 128 + row;
@@ -108,22 +101,20 @@ __device__ __forceinline__ void epilogue_qkv(const GemmArgs& g, int tile, int ro
     if (col < g.n_out) {
 #pragma unroll 1
         for (int j = 0; j < nj; ++j) {
-            const int pos = live ? row_pos[jb + j] : 0;
+            const int pos = live ? row_pos[j] : 0;
             if (pos < 0) continue;
             float val = stage[row][j];
             if (mat < 2) {
-                const float2 cs = rope_s ? rope_s[j * half + fi]
-                                         : make_float2(__ldg(&g.rope_cos[(int64_t)pos * half + fi]),
-                                                       __ldg(&g.rope_sin[(int64_t)pos * half + fi]));
+                const float2 cs = rope_s[j * half + fi];
                 const float other = stage[prow][j];
                 val = lower ? (val * cs.x - other * cs.y) : (other * cs.y + val * cs.x);
             }
             if (!live) continue;
             if (mat == 0) {
-                g.out_f32[(int64_t)(jb + j) * g.ld + col] = val;
+                g.out_f32[(int64_t)j * g.ld + col] = val;
             } else {
                 __nv_bfloat16* cache = mat == 1 ? g.kcache : g.vcache;
-                cache[kv_row_index(d, g.layer, row_seq[jb + j], head, pos) * hd + idx] = __float2bfloat16_rn(val);
+                cache[kv_row_index(d, g.layer, row_seq[j], head, pos) * hd + idx] = __float2bfloat16_rn(val);
             }
         }
     }
@@ -131,15 +122,14 @@ __device__ __forceinline__ void epilogue_qkv(const GemmArgs& g, int tile, int ro
 }
 
 // SwiGLU: tile rows 0..63 are gate features, 64..127 the matching up features.
-__device__ __forceinline__ void epilogue_swiglu(const GemmArgs& g, int tile, int row, int jb, int nj,
-                                                float (*stage)[33], bool live) {
+__device__ __forceinline__ void epilogue_swiglu(const GemmArgs& g, int tile, int row, int nj, float (*stage)[33], bool live) {
     const int fi = row & 63, f = tile * 64 + fi;
     if (f < g.n_out) {
 #pragma unroll 1
         for (int j = row >> 6; j < nj; j += 2) {
             const float gate = stage[g.gate_second ? 64 + fi : fi][j], up = stage[g.gate_second ? fi : 64 + fi][j];
             const float v = gate / (1.f + expf(-gate)) * up;
-            if (live) store_act(g.out_act, kActSplit, g.rc, jb + j, f, g.n_out, v);
+            if (live) store_split(g.out_act, g.rc, j, f, g.n_out, v);
         }
     }
     epi_sync();
@@ -148,8 +138,8 @@ __device__ __forceinline__ void epilogue_swiglu(const GemmArgs& g, int tile, int
 // LM head: optional logits store, then the tile's (max, lowest argmax) for every used row.  Row-major like the
 // epilogues above: thread t takes activation row j = t & 31 and 32 consecutive features, so a row costs no shuffles
 // (five steps of two per row before: 25 us per 144-row tile, 3 us at nine rows).
-__device__ __forceinline__ void epilogue_lmhead(const GemmArgs& g, int tile, int t, int jb, int nj,
-                                                float (*stage)[33], float* red_f, int* red_i, bool live) {
+__device__ __forceinline__ void epilogue_lmhead(const GemmArgs& g, int tile, int t, int nj, float (*stage)[33], float* red_f, int* red_i,
+                                                bool live) {
     const int j = t & 31, w = t >> 5, f0 = 32 * w;
     const int v0 = tile * 128 + f0, nv = min(32, g.n_out - v0);  // nv <= 0: past the vocabulary
     if (j < nj) {
@@ -170,7 +160,7 @@ __device__ __forceinline__ void epilogue_lmhead(const GemmArgs& g, int tile, int
         red_f[w * 32 + j] = bv;
         red_i[w * 32 + j] = bi;
         if (g.out_f32 && live) {
-            float* o = g.out_f32 + (int64_t)(jb + j) * g.ld + v0;
+            float* o = g.out_f32 + (int64_t)j * g.ld + v0;
             if (nv == 32 && (g.ld & 3) == 0) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
@@ -189,8 +179,8 @@ __device__ __forceinline__ void epilogue_lmhead(const GemmArgs& g, int tile, int
         for (int u = 1; u < 4; ++u)  // ascending features: the lowest index on ties
             if (red_f[u * 32 + j] > bv) { bv = red_f[u * 32 + j]; bi = red_i[u * 32 + j]; }
         if (live) {
-            g.part_max[(int64_t)tile * g.rc + jb + j] = bv;
-            g.part_idx[(int64_t)tile * g.rc + jb + j] = bi;
+            g.part_max[(int64_t)tile * g.rc + j] = bv;
+            g.part_idx[(int64_t)tile * g.rc + j] = bi;
         }
     }
     epi_sync();
@@ -337,19 +327,18 @@ __device__ __forceinline__ void block_qkv(const GemmArgs& g, int tile, int warp,
     sync();
 }
 
-// h = silu(gate) * up: half a warp per row; n_out % 64 == 0
+// h = silu(gate) * up, the tile's features 0..63 and 64..127: half a warp per row; n_out % 64 == 0
 template <typename Sync>
 __device__ __forceinline__ void block_swiglu(const GemmArgs& g, int tile, int warp, int lane, int jb, int nj, float (*st)[kBlockLd],
                                              Sync sync) {
     const int f = 4 * (lane & 15);
-    const int gate_at = g.gate_second ? 64 : 0, up_at = 64 - gate_at;
     __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(g.out_act) + (int64_t)jb * g.n_out + tile * 64 + f;
     const int64_t lo_term = (int64_t)g.rc * g.n_out;
     sync();
     auto row = [&](int u) {
         const int j = 2 * (warp + 4 * u) + (lane >> 4);
-        const float4 a = *reinterpret_cast<const float4*>(&st[j][gate_at + f]);
-        const float4 b = *reinterpret_cast<const float4*>(&st[j][up_at + f]);
+        const float4 a = *reinterpret_cast<const float4*>(&st[j][f]);
+        const float4 b = *reinterpret_cast<const float4*>(&st[j][64 + f]);
         const float4 v = make_float4(a.x / (1.f + expf(-a.x)) * b.x, a.y / (1.f + expf(-a.y)) * b.y, a.z / (1.f + expf(-a.z)) * b.z,
                                      a.w / (1.f + expf(-a.w)) * b.w);
         if (j < nj) store_split4(h + (int64_t)j * g.n_out, lo_term, v);

@@ -318,11 +318,10 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
         // ------------------------------- epilogue warps ------------------------------------------
         const int row = threadIdx.x;  // 0..127 = TMEM lane = output feature inside the tile
         int rows_used = 0;
-        constexpr bool kPrefetchX = true;
         // residual rows of a tile: requested early, so their latency hides behind the accumulator wait
         // and the cross-CTA sum (only the tile's owner ever writes them, in its epilogue)
         auto prefetch_x = [&](int tile, float (&xpre)[kXPre]) {
-            if (kPrefetchX && MODE == kGemmResid) {
+            if (MODE == kGemmResid) {
                 const int col = tile * 128 + row;
 #pragma unroll
                 for (int u = 0; u < kXPre - 1; ++u)
@@ -341,11 +340,11 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
                 for (int j = 0; j < NR; ++j) stage[row][j] = acc[j];
             }
             epi_sync();
-            if constexpr (MODE == kGemmQKV) epilogue_qkv(g, tile, row, 0, nj, stage, red_i, red_i + 32, rope_s, live);
-            else if constexpr (MODE == kGemmResid) epilogue_resid<kPrefetchX>(g, tile, row, 0, nj, stage, red_f, xpre, live);
-            else if constexpr (MODE == kGemmSwiGLU) epilogue_swiglu(g, tile, row, 0, nj, stage, live);
-            else if constexpr (MODE == kGemmStore) epilogue_store(g, tile, row, 0, rows_used, stage);
-            else epilogue_lmhead(g, tile, row, 0, nj, stage, red_f, red_i, live);
+            if constexpr (MODE == kGemmQKV) epilogue_qkv(g, tile, row, nj, stage, red_i, red_i + 32, rope_s, live);
+            else if constexpr (MODE == kGemmResid) epilogue_resid(g, tile, row, nj, stage, xpre, live);
+            else if constexpr (MODE == kGemmSwiGLU) epilogue_swiglu(g, tile, row, nj, stage, live);
+            else if constexpr (MODE == kGemmStore) epilogue_store(g, tile, row, rows_used, stage);
+            else epilogue_lmhead(g, tile, row, nj, stage, red_f, red_i, live);
         };
         // Tiles cut by a range boundary.  The CTA whose range holds the tile's FIRST chunks owns it: that is
         // the last thing it works on, so it completes the tile at once.  Every other CTA of the tile hands its
@@ -356,7 +355,6 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
         // before the owner asks: a tile cut in two costs its owner no wait at all; only CTAs whose whole range
         // lies inside one tile finish together with the owner.
         constexpr uint32_t kEmpty = 0xFFFFFFFFu;
-        bool aborted = false;
         int seg;
         asm volatile("mov.s32 %0, -1;" : "=r"(seg));  // segment -1: the turn without loads and stores (opaque: one copy of the code)
 #pragma unroll 1
@@ -410,7 +408,7 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
             }
             epi_sync();
             const bool ok = !live || sh[2 + buf] != 0;
-            if (!ok) { aborted = true; break; }
+            if (!ok) break;
             if (threadIdx.x == 0 && live) LLMA_STAMP(stp, 4);
             tc_fence_after();
             float acc[32];
@@ -501,7 +499,6 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
             finish_tile(tile, acc, xpre, live);
             tile += live ? 1 : 0;
         }
-        (void)aborted;
         if (threadIdx.x == 0) LLMA_STAMP(stp, 5);
     }
     tc_fence_before();

@@ -2,7 +2,7 @@
 //
 //   out[r, n] = sum_k W[n, k] * a[r, k],  r < rows (up to 256 activation rows), W bf16 [n_out, k_in].
 //
-// The activations arrive split into two bf16 terms (ActLayout kActSplit: hi rows, then lo rows); both
+// The activations arrive split into two bf16 terms (hi rows, then lo rows); both
 // are multiplied by the same weight tile and summed in fp32, so the product keeps 16 mantissa bits
 // of the activations at no cost in weight traffic.
 //
@@ -38,7 +38,7 @@ struct GemmArgs {
     int32_t chunks;         // k_in / 64
     int32_t tiles_per_map;  // tiles per A map
     const RowDesc* rows;    // nullptr: all nr rows are in use
-    const void* act;        // activation operand, ActLayout kActSplit [2 rc][k_in] bf16
+    const void* act;        // activation operand, split bf16 [2 rc][k_in]
     int32_t rc;             // row capacity of the activation buffers and per-row scratch arrays
     int32_t nr;             // rows the launch is shaped for (wide kernel: multiple of 16, <= 256)
     unsigned long long* stamps;  // measurement builds: timeline block (see LLMA_STAMPS), else unused
@@ -50,8 +50,8 @@ struct GemmArgs {
     int32_t* dev_err;
     float* out_f32;         // Resid: x; QKV: qkv buffer; LmHead: logits or nullptr
     int32_t ld;             // leading dimension of out_f32
-    void* out_act;          // SwiGLU: h in ActLayout kActSplit [2 rc][d_ffn]
-    int32_t gate_second;    // SwiGLU: 1 when the tile's rows 0..63 are the up features and 64..127 the gate features
+    void* out_act;          // SwiGLU: h, split bf16 [2 rc][d_ffn]
+    int32_t gate_second;    // SwiGLU, gemm_ws_kernel: 1 when the tile's rows 0..63 are the up features and 64..127 the gate features
     // RMSNorm folded into the projections: the producer of the residual stream x writes
     // xs = split(x * gain) and, per 128-column tile, the rows' sums of squares; the consumer
     // multiplies its accumulators by rsqrt(sum / norm_dim + eps), which equals projecting the
@@ -61,7 +61,7 @@ struct GemmArgs {
     float norm_inv;         // 1 / features of a row
     float norm_eps;
     const float* gain_next; // Resid producer: gain of the next norm [n_out], with xs_out / ss_out
-    void* xs_out;           // ActLayout kActSplit [2 rc][n_out], or nullptr
+    void* xs_out;           // split bf16 [2 rc][n_out], or nullptr
     float* ss_out;          // [n_tiles][rc]
     // QKV
     ModelDims dims;
@@ -110,11 +110,10 @@ template <int NR, int MODE> struct GemmCfg {
 // Bytes of gemm_ws_kernel's hand-over slots for a grid of up to `ctas` CTAs
 constexpr size_t gemm_ws_bytes(int ctas) { return (size_t)ctas * 128 * 32 * sizeof(float); }
 
-// Shared-memory plan of gemm_wide_kernel for nr rows: a ring of weight tiles (16 KB each) and a ring of
-// activation tiles (nr rows of 128 bytes each: one term of one 64-wide k-chunk), as many as fit.
+// Shared-memory plan of gemm_wide_kernel for nr rows: a ring of stages, each a weight tile (16 KB) and the two terms' nr rows
+// of one 64-wide k-chunk, as many as fit.
 struct GemmWideCfg {
-    uint32_t b_slot;    // bytes of one activation tile: nr rows of 128 bytes for each of the two terms
-    int sa, sb;         // ring depths (each at most 8)
+    int stages;         // ring depth (at most 8)
     uint32_t tmem_cols; // power of two >= the accumulators' columns (2 nr each; two of them up to 128 rows, else one)
     size_t smem_bytes;
 };

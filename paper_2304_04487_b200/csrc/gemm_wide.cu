@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kGemmWideThreads, 1)
 gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                  const __grid_constant__ CUtensorMap map_a2, const __grid_constant__ CUtensorMap map_b0,
                  const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_b2,
-                 const __grid_constant__ CUtensorMap map_b3, const int SA, const uint32_t tmem_cols) {
+                 const __grid_constant__ CUtensorMap map_b3, const int S, const uint32_t tmem_cols) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* gen_base = smem_raw + (base - smem_u32(smem_raw));
@@ -59,21 +59,19 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
         return i;
     };
     const uint32_t sA = base, sB = base + kGemmABytes;   // stage s: sA + s * stage_bytes, sB + s * stage_bytes
-    uint8_t* after = gen_base + (size_t)SA * stage_bytes;
+    uint8_t* after = gen_base + (size_t)S * stage_bytes;
     float (*stage)[kBlockLd] = reinterpret_cast<float (*)[kBlockLd]>(after);
     uint8_t* tail = after + kWideStageBytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);  // full[8], empty[8], (16 unused), acc_full[2], acc_empty[2]
-    volatile uint32_t* sh = reinterpret_cast<volatile uint32_t*>(tail + 36 * 8);  // [0] TMEM base, [1] abort, [2] broadcast
-    float* rscale = reinterpret_cast<float*>(tail + 36 * 8 + 16);                 // [256] per-row norm scales
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);  // full[8], empty[8], acc_full[2], acc_empty[2]
+    volatile uint32_t* sh = reinterpret_cast<volatile uint32_t*>(tail + 20 * 8);  // [0] TMEM base, [1] abort, [2] broadcast
+    float* rscale = reinterpret_cast<float*>(tail + 20 * 8 + 16);                 // [256] per-row norm scales
     int* s_pos = reinterpret_cast<int*>(rscale + kRowCap);                                                     // [256] (QKV mode)
     int* s_seq = s_pos + kRowCap;                                                 // [256]
     const uint32_t bar0 = smem_u32(bars);
-    auto full_a = [&](int s) { return bar0 + 8u * s; };
-    auto empty_a = [&](int s) { return bar0 + 8u * (8 + s); };
-    auto full_b = full_a;    // both halves of a stage land on one barrier (two arrivals with their byte counts)
-    auto empty_b = empty_a;  // and are released together
-    auto accf_bar = [&](int i) { return bar0 + 8u * (32 + i); };
-    auto acce_bar = [&](int i) { return bar0 + 8u * (34 + i); };
+    auto full_bar = [&](int s) { return bar0 + 8u * s; };  // both halves of a stage: two arrivals with their byte counts
+    auto empty_bar = [&](int s) { return bar0 + 8u * (8 + s); };
+    auto accf_bar = [&](int i) { return bar0 + 8u * (16 + i); };
+    auto acce_bar = [&](int i) { return bar0 + 8u * (18 + i); };
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int G = gridDim.x, b = blockIdx.x;
@@ -91,7 +89,7 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
     if (threadIdx.x == 0) LLMA_STAMP(stp, 0);
     if (threadIdx.x == 0) {
         for (int s = 0; s < 8; ++s) {
-            mbar_init(full_a(s), 2); mbar_init(empty_a(s), 1);
+            mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1);
         }
         for (int i = 0; i < 2; ++i) { mbar_init(accf_bar(i), 1); mbar_init(acce_bar(i), 4); }
         sh[1] = 0; sh[2] = 0;
@@ -126,23 +124,23 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
             uint32_t ph = 0;
 #pragma unroll 1
             for (; it < n_items && !sh[1]; ++it) {
-                if (it >= SA && !mbar_wait(empty_a(s), ph ^ 1u)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
-                mbar_arrive_expect_tx(full_a(s), kGemmABytes);
+                if (it >= S && !mbar_wait(empty_bar(s), ph ^ 1u)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
+                mbar_arrive_expect_tx(full_bar(s), kGemmABytes);
                 const uint32_t dstA = sA + (uint32_t)s * stage_bytes;
                 if (MODE == kGemmSwiGLU) {
-                    tma_load_2d(dstA, &map_a0, full_a(s), c * 64, tile * 64);
-                    tma_load_2d(dstA + kGemmABytes / 2, &map_a1, full_a(s), c * 64, tile * 64);
+                    tma_load_2d(dstA, &map_a0, full_bar(s), c * 64, tile * 64);
+                    tma_load_2d(dstA + kGemmABytes / 2, &map_a1, full_bar(s), c * 64, tile * 64);
                 } else {
                     const CUtensorMap* mp = m == 0 ? &map_a0 : (m == 1 ? &map_a1 : &map_a2);
-                    tma_load_2d(dstA, mp, full_a(s), c * 64, rt * 128);
+                    tma_load_2d(dstA, mp, full_bar(s), c * 64, rt * 128);
                 }
                 if (++c == C) { c = 0; ++tile; if (++rt == g.tiles_per_map) { rt = 0; ++m; } }
-                if (++s == SA) { s = 0; ph ^= 1u; }
+                if (++s == S) { s = 0; ph ^= 1u; }
             }
             if (sh[1]) {  // give up: let the copies already issued land before the CTA's memory goes away
 #pragma unroll 1
-                for (int j = it - 1; j >= 0 && j >= it - SA; --j)
-                    (void)mbar_wait(full_a(j % SA), (uint32_t)((j / SA) & 1), 100000000ull);
+                for (int j = it - 1; j >= 0 && j >= it - S; --j)
+                    (void)mbar_wait(full_bar(j % S), (uint32_t)((j / S) & 1), 100000000ull);
             }
         }
     } else if (warp == 6) {
@@ -158,16 +156,16 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
             uint32_t ph = 0;
 #pragma unroll 1
             for (; q < n_items && !sh[1]; ++q) {
-                if (q >= SA && !mbar_wait(empty_b(s), ph ^ 1u)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
-                mbar_arrive_expect_tx(full_b(s), b_slot);
-                tma_load_3d(sB + (uint32_t)s * stage_bytes, map_b, full_b(s), c * 64, 0, 0);
+                if (q >= S && !mbar_wait(empty_bar(s), ph ^ 1u)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
+                mbar_arrive_expect_tx(full_bar(s), b_slot);
+                tma_load_3d(sB + (uint32_t)s * stage_bytes, map_b, full_bar(s), c * 64, 0, 0);
                 if (++c == C) c = 0;
-                if (++s == SA) { s = 0; ph ^= 1u; }
+                if (++s == S) { s = 0; ph ^= 1u; }
             }
             if (sh[1]) {
 #pragma unroll 1
-                for (int j = q - 1; j >= 0 && j >= q - SA; --j)
-                    (void)mbar_wait(full_b(j % SA), (uint32_t)((j / SA) & 1), 100000000ull);
+                for (int j = q - 1; j >= 0 && j >= q - S; --j)
+                    (void)mbar_wait(full_bar(j % S), (uint32_t)((j / S) & 1), 100000000ull);
             }
         }
     } else if (warp == 5) {
@@ -192,9 +190,8 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
             uint32_t s_ph = 0;    // run-time ring depth would cost this thread more than a commit
             int seg = 0;
 #ifdef LLMA_STAMPS
-            // measurement build: time this thread spends waiting for weight stages (word 6) and for activation
-            // slots (word 7), in ns
-            unsigned long long wait_a = 0, wait_b = 0, tw;
+            // measurement build: time this thread spends waiting for ring stages (word 6), in ns
+            unsigned long long wait_a = 0, tw;
 #define LLMA_WAIT_BEGIN() (tw = globaltimer_ns())
 #define LLMA_WAIT_END(acc) (acc += globaltimer_ns() - tw)
 #else
@@ -212,7 +209,7 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
 #pragma unroll 1
                 for (int c = c0; c < c1 && !sh[1]; ++c, ++ia) {
                     LLMA_WAIT_BEGIN();
-                    if (!mbar_wait(full_a(s), s_ph)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
+                    if (!mbar_wait(full_bar(s), s_ph)) { atomicExch(g.dev_err, kDevErrTimeout); sh[1] = 1; break; }
                     LLMA_WAIT_END(wait_a);
                     if (ia == 0) LLMA_STAMP(stp, 2);
                     tc_fence_after();
@@ -225,8 +222,8 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
                         umma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (acc_on || kk > 0) ? 1u : 0u);
                         if (!one_mma) umma_bf16(d_tmem + (uint32_t)nr, da + 2 * kk, db_lo + 2 * kk, idesc, (acc_on || kk > 0) ? 1u : 0u);
                     }
-                    umma_commit(empty_a(s));  // the stage is free once these MMAs have read it
-                    if (++s == SA) { s = 0; s_ph ^= 1u; }
+                    umma_commit(empty_bar(s));  // the stage is free once these MMAs have read it
+                    if (++s == S) { s = 0; s_ph ^= 1u; }
                 }
                 if (sh[1]) break;
                 umma_commit(accf_bar(buf));  // accumulator complete
@@ -234,7 +231,7 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
                 w += c1 - c0;
             }
 #ifdef LLMA_STAMPS
-            if (stp) { stp[6] = wait_a; stp[7] = wait_b; }
+            if (stp) stp[6] = wait_a;
 #endif
         }
     } else {
@@ -442,12 +439,11 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
 // ---- host side ------------------------------------------------------------------------------------
 GemmWideCfg gemm_wide_cfg(int nr) {
     GemmWideCfg c;
-    c.b_slot = (uint32_t)nr * 256u;
     const size_t budget = (size_t)227 * 1024 - 1024 - kWideStageBytes - kWideTailBytes;
-    const size_t stage_bytes = kGemmABytes + c.b_slot;
+    const size_t stage_bytes = kGemmABytes + (size_t)nr * 256;
     int S = (int)(budget / stage_bytes);  // as many stages as fit, at most 8
     if (S > 8) S = 8;
-    c.sa = c.sb = S;
+    c.stages = S;
     uint32_t cols = 32;
     for (int i = 0; i < 4; ++i) {  // the largest need over the row counts a step may choose (as in the kernel)
         const uint32_t acc_cols = 2u * (uint32_t)wide_box_rows(nr, i);
@@ -485,13 +481,13 @@ void launch_gemm_wide(cudaStream_t st, int grid, bool pdl, const GemmArgs& args,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    const int sa = c.sa;
+    const int stages = c.stages;
     const uint32_t cols = c.tmem_cols;
     switch (args.mode) {
-        case kGemmQKV: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmQKV>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], sa, cols); break;
-        case kGemmResid: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmResid>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], sa, cols); break;
-        case kGemmSwiGLU: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmSwiGLU>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], sa, cols); break;
-        default: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmLmHead>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], sa, cols); break;
+        case kGemmQKV: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmQKV>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], stages, cols); break;
+        case kGemmResid: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmResid>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], stages, cols); break;
+        case kGemmSwiGLU: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmSwiGLU>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], stages, cols); break;
+        default: cudaLaunchKernelEx(&cfg, gemm_wide_kernel<kGemmLmHead>, args, a0, a1, a2, map_b[0], map_b[1], map_b[2], map_b[3], stages, cols); break;
     }
 }
 

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(128) embed_norm_kernel(ModelDims dims, const R
     if (col < d) {
         v = ok ? __bfloat162float(er[col]) : 0.f;
         x[(int64_t)r * d + col] = v;
-        store_act(xs, kActSplit, dims.row_cap, r, col, d, v * gain[col]);
+        store_split(xs, dims.row_cap, r, col, d, v * gain[col]);
     }
     float sq = v * v;
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -364,10 +364,10 @@ __global__ void __launch_bounds__(128) embed_prompt_kernel(int d, int rc, const 
         const int col = t * 128 + lane * 4;
         const float4 v = load4_each(er + col), gn = load4_each(gain + col);
         *reinterpret_cast<float4*>(x + (int64_t)r * d + col) = v;
-        store_act(xs, kActSplit, rc, r, col, d, v.x * gn.x);
-        store_act(xs, kActSplit, rc, r, col + 1, d, v.y * gn.y);
-        store_act(xs, kActSplit, rc, r, col + 2, d, v.z * gn.z);
-        store_act(xs, kActSplit, rc, r, col + 3, d, v.w * gn.w);
+        store_split(xs, rc, r, col, d, v.x * gn.x);
+        store_split(xs, rc, r, col + 1, d, v.y * gn.y);
+        store_split(xs, rc, r, col + 2, d, v.z * gn.z);
+        store_split(xs, rc, r, col + 3, d, v.w * gn.w);
         float sq = (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
         for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
         if (lane == 0) ss[(int64_t)t * rc + r] = sq;

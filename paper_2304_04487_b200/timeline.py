@@ -9,8 +9,8 @@ Needs the measurement build of the library (it records nothing otherwise):
 Prints, per projection of a layer (averaged over the inner layers of the last step of a decode), the
 events of its CTAs relative to the end of the projection before it, and what the attention kernels
 between the QKV and the output projection do.  All times in microseconds.  With --batch B the B sequences
-decode together; beyond 32 rows per step that is the wide GEMM kernel, whose last two words per CTA are the
-time its MMA thread spent waiting for ring stages and (unused) zero.
+decode together; beyond 32 rows per step that is the wide GEMM kernel, whose last word per CTA is the
+time its MMA thread spent waiting for ring stages.
 """
 from __future__ import annotations
 
