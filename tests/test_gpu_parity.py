@@ -482,11 +482,11 @@ def test_cuda_core_widths(d, heads, hd, ffn, vocab, dtype, k, B):
     eng.llma_destroy()
 
 
-# ---- long prompt passes: shortest one, one row past a tile, several passes, odd numbers of feature tiles -------------
+# ---- prompt passes of narrow decoders (tiles of 64 rows): rows past a tile, several passes, odd numbers of feature tiles ----
 @pytest.mark.parametrize("d,heads,hd,ffn,P", [
-    (256, 4, 64, 1024, 161),                     # 160 rows: the shortest long pass
+    (256, 4, 64, 1024, 161),                     # 160 rows: two tiles and a half
     (384, 3, 128, 448, 162),                     # 9, 3 and 7 tiles of 128 features: the odd CTA of a pair idles
-    (384, 3, 128, 448, 322),                     # one row past five tiles of 64
+    (384, 3, 128, 448, 322),                     # one row past five tiles
     (256, 2, 128, 576, 2200)])                   # 2199 rows: two passes, the second against the first one's cache
 def test_long_prompt_passes(d, heads, hd, ffn, P):
     shape = ModelShape(f"prompt-{d}-{hd}-{ffn}", 2, d, heads, hd, ffn, 1000, "bf16")
