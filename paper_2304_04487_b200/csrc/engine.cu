@@ -59,7 +59,7 @@ static void free_engine(llma_engine* e) {
     cudaFree(e->rope_cos); cudaFree(e->rope_sin); cudaFree(e->kcache); cudaFree(e->vcache);
     cudaFree(e->attn_ws_o); cudaFree(e->attn_ws_ml); cudaFree(e->trace); cudaFree(e->target);
     cudaFree(e->gemm_ws); cudaFree(e->stamps); cudaFree(e->gemm_ws_wide); cudaFree(e->gemm_flags); cudaFree(e->part_max); cudaFree(e->part_idx); cudaFree(e->norm_ss);
-    cudaFree(e->p_tok);
+    cudaFree(e->p_tok); cudaFree(e->step_ops); cudaFree(e->grid_barrier); cudaFree(e->ll_words);
     free_prompt_buffers(e);
     if (e->h_block) cudaFreeHost(e->h_block);
     for (int i = 0; i < 2; ++i)
@@ -83,6 +83,41 @@ static cudaError_t alloc_prompt_buffers(llma_engine* e) {
     if (r == cudaSuccess) r = dalloc((char**)&e->p_h, rows * d.d_ffn * 4);
     if (r != cudaSuccess) free_prompt_buffers(e);
     return r;
+}
+
+// Whole decoding steps of the CUDA-core path in one launch, where the rows of a pass fit shared memory
+static cudaError_t init_whole_steps(llma_engine* e) {
+    const ModelDims& d = e->dims;
+    int coop = 0;
+    cudaError_t r = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, e->device);
+    if (r != cudaSuccess) return r;
+    SimtStep& s = e->simt;
+    bool fits = false;
+    if (!coop || !step_simt_shape(d, e->bf16, e->y_cap, e->num_sms, &s, &e->simt_smem)) return cudaSuccess;
+    r = init_step_simt(e->bf16, d.head_dim, e->simt_smem, &fits);
+    if (r != cudaSuccess || !fits) return r;
+    std::vector<SimtOp> ops;
+    for (int l = 0; l < d.n_layers; ++l) {
+        ops.push_back({e->wq[l], e->wk[l], e->wv[l], e->attn_norm[l]});
+        ops.push_back({e->wo[l], nullptr, nullptr, nullptr});
+        ops.push_back({e->w_gate[l], e->w_up[l], nullptr, e->ffn_norm[l]});
+        ops.push_back({e->w_down[l], nullptr, nullptr, nullptr});
+    }
+    ops.push_back({e->lm_head, nullptr, nullptr, e->final_norm});
+    if ((r = dalloc(&e->step_ops, ops.size(), false)) != cudaSuccess) return r;
+    if ((r = cudaMemcpy(e->step_ops, ops.data(), ops.size() * sizeof(SimtOp), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
+    if ((r = dalloc(&e->grid_barrier, 1)) != cudaSuccess) return r;
+    const size_t rc = (size_t)e->row_cap, parts = 2 * (size_t)e->num_sms * rc;
+    e->ll_count = rc * (d.d_model + 4 * (size_t)d.hd_total + d.d_ffn) + parts + simt_rows_words(e->row_cap);
+    if ((r = dalloc(&e->ll_words, e->ll_count)) != cudaSuccess) return r;
+    s.ll_x = e->ll_words; s.ll_qkv = s.ll_x + rc * d.d_model; s.ll_attn = s.ll_qkv + rc * 3 * d.hd_total;
+    s.ll_h = s.ll_attn + rc * d.hd_total; s.ll_part = s.ll_h + rc * d.d_ffn; s.ll_rows = s.ll_part + parts;
+    s.dims = d; s.ops = e->step_ops; s.emb = e->tok_emb; s.rows = e->rows;
+    s.x = e->x; s.qkv = e->qkv; s.attn = (float*)e->attn; s.h = (float*)e->h; s.logits = e->cfg.keep_logits ? e->logits : nullptr;
+    s.kcache = e->kcache; s.vcache = e->vcache; s.rope_cos = e->rope_cos; s.rope_sin = e->rope_sin;
+    s.barrier = e->grid_barrier; s.dev_err = e->dev_err;
+    e->step_simt = true;
+    return cudaSuccess;
 }
 
 extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* cuda_stream, llma_engine** out) {
@@ -203,7 +238,10 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     const size_t parts_max = std::max<size_t>(vt, (size_t)2 * e->num_sms);
     CREATE_TRY(dalloc(&e->part_max, parts_max * RC));
     CREATE_TRY(dalloc(&e->part_idx, parts_max * RC));
-    if (e->gemm_impl != LLMA_GEMM_TCGEN05) CREATE_TRY(init_rowgemm(e->bf16));
+    if (e->gemm_impl != LLMA_GEMM_TCGEN05) {
+        CREATE_TRY(init_rowgemm(e->bf16));
+        CREATE_TRY(init_whole_steps(e));
+    }
     if (e->gemm_impl == LLMA_GEMM_TCGEN05) {
         int major = 0;
         CREATE_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));

@@ -8,6 +8,7 @@
 #include "attention_mma.cuh"
 #include "gemm_tcgen05.cuh"
 #include "kernels.h"
+#include "step_simt.cuh"
 
 struct llma_engine {
     llma_config cfg;
@@ -77,6 +78,16 @@ struct llma_engine {
     int attn_tiles = 1;             // 128-position tiles per attention CTA in decoding steps (a function of the capacity only)
     float *attn_ws_o = nullptr, *attn_ws_ml = nullptr;
 
+    // whole steps in one cooperative launch: CUDA-core path (step_simt.cu)
+    bool step_simt = false;
+    llma::SimtStep simt{};          // everything that does not change from launch to launch
+    size_t simt_smem = 0;
+    llma::SimtOp* step_ops = nullptr;
+    uint32_t* grid_barrier = nullptr;
+    unsigned long long* ll_words = nullptr;   // activations on their way from CTA to CTA
+    size_t ll_count = 0;
+    uint32_t ll_epoch = 1;                    // first number of the next launch
+
     // replay of a given step sequence (llma_generate_forced)
     int32_t *trace = nullptr, *target = nullptr;
     int32_t trace_cap = 0;
@@ -119,6 +130,9 @@ constexpr size_t kStepGraphs = 64;     // n is any positive number: the pair use
 // llma_step launches kernel by kernel until an (n, k) has been used this often: capturing a step costs what a graph saves in 12 to
 // 23 of them (two layers of width 1024 115 against 10 us, three of width 512 170 against 8, the 7B shape 1400 against 60).
 constexpr int kCaptureAt = 16;
+// Steps of one launch of a whole-step kernel, which ends by itself once there is nothing left to do: enough that launching costs
+// nothing (5 us against 32 steps of 20 us and more), few enough that other streams get the GPU every millisecond or so.
+constexpr int kStepsPerLaunch = 32;
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date
 void gemm_count_engine(int dev, int by);  // the last engine of a device takes the scratch that llma_gemm_rows32_bf16 keeps with it

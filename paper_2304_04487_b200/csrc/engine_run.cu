@@ -169,17 +169,22 @@ static void enqueue_embed(llma_engine* e) {
 
 // the integer kernel between forward passes: acceptance + K/V commit of the pass that has finished,
 // trigger search + copy + row packing for the one that follows
-static void enqueue_tail(llma_engine* e, int n, int k, bool accept, bool plan) {
+static TailArgs tail_args(const llma_engine* e, int n, int k) {
     TailArgs t;
     std::memset(&t, 0, sizeof(t));
     t.dims = e->dims; t.st = e->seq_state; t.rows = e->rows; t.ref = e->ref; t.y = e->y; t.y_cap = e->y_cap; t.n = n; t.k = k;
-    t.do_accept = accept ? 1 : 0; t.do_plan = plan ? 1 : 0;
     t.part_max = e->part_max; t.part_idx = e->part_idx;
     t.n_tiles = e->gemm_impl == LLMA_GEMM_TCGEN05 ? (e->dims.vocab + 127) / 128
                                                   : rowgemm_grid((e->dims.vocab + 1) / 2, e->dims.d_model, row_bound(e, true), e->num_sms);
     t.out_tok = e->out_tok; t.n_rows = e->decode_rows;
     t.trace = e->trace; t.target = e->target; t.trace_cap = e->trace_cap;
     t.dev_err = e->dev_err;
+    return t;
+}
+
+static void enqueue_tail(llma_engine* e, int n, int k, bool accept, bool plan) {
+    TailArgs t = tail_args(e, n, k);
+    t.do_accept = accept ? 1 : 0; t.do_plan = plan ? 1 : 0;
     launch_step_tail(e->stream, t);
     mark(e, accept ? LLMA_K_ACCEPT : LLMA_K_PLAN);
     e->launch_counter += 1;
@@ -195,6 +200,28 @@ static void enqueue_step_body(llma_engine* e, int n, int k, bool plan_next) {
     e->launch_counter += 1;
     enqueue_forward(e, true);
     enqueue_tail(e, n, k, true, plan_next);
+}
+
+// Up to `steps` decoding steps as launches of the whole-step kernel (fewer if no sequence has anything left to do).  plan_first: plan
+// the first one (otherwise the launch before has planned it); plan_last: plan the step after the last one.
+static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps, bool plan_first, bool plan_last) {
+    SimtStep s = e->simt;
+    s.tail = tail_args(e, n, k);
+    const uint32_t per_step = simt_epochs(e->dims);
+    for (; steps > 0; steps -= kStepsPerLaunch, plan_first = false) {
+        s.max_steps = std::min(steps, kStepsPerLaunch);
+        s.plan_first = plan_first ? 1 : 0;
+        s.plan_last = plan_last || steps > kStepsPerLaunch ? 1 : 0;
+        if (e->ll_epoch > 0xFFFFFFFFu - per_step * (kStepsPerLaunch + 2)) {  // the numbers begin again
+            CU_TRY(cudaMemsetAsync(e->ll_words, 0, e->ll_count * sizeof(unsigned long long), e->stream));
+            e->ll_epoch = 1;
+        }
+        s.epoch = e->ll_epoch;
+        e->ll_epoch += per_step * (uint32_t)(s.max_steps + 1);  // (the rows of the step after the last one are published too)
+        CU_TRY(launch_step_simt(e->stream, e->bf16, s, e->simt_smem, e->num_sms));
+        e->launch_counter += 1;
+    }
+    return LLMA_OK;
 }
 
 // The state on its way to and from the device.  Every call that launches kernels brings the mirror up to date, uploads
@@ -241,7 +268,7 @@ static int check_device_error(llma_engine* e) {
     // a kernel that gave up may have left partial tiles in the hand-over slots: empty them again, so that
     // a caller who carries on after the error does not sum stale partials into later projections
     if (code == kDevErrTimeout && e->gemm_ws) CU_TRY(cudaMemsetAsync(e->gemm_ws, 0xFF, e->gemm_ws_bytes, e->stream));
-
+    if (code == kDevErrTimeout && e->grid_barrier) CU_TRY(cudaMemsetAsync(e->grid_barrier, 0, sizeof(uint32_t), e->stream));
     CU_TRY(cudaStreamSynchronize(e->stream));
     *e->h_err = kDevErrNone;
     if (code == kDevErrTimeout) return LLMA_ERR_DEVICE_TIMEOUT;
@@ -438,6 +465,7 @@ static int capture(llma_engine* e, cudaGraphExec_t* out, Enqueue enqueue) {
 }
 
 static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
+    if (e->step_simt) return enqueue_whole_steps(e, n, k, 1, true, false);
     auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
     llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k);
     if (!e->can_capture || g.uses + 1 < kCaptureAt) {
@@ -562,20 +590,24 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         S.done = max_new == 0;
         e->state_dirty = true;
     }
+    const bool whole = e->step_simt;
     cudaGraphExec_t graph = nullptr;
-    rc = get_step_graph(e, n, k, &graph);
-    if (rc) return rc;
+    if (!whole) {
+        rc = get_step_graph(e, n, k, &graph);
+        if (rc) return rc;
+    }
 
     rc = push_state(e);
     if (rc) return rc;
 
     // Each step emits between 1 and k+1 tokens per sequence, so ceil(left / (k+1)) more steps
     // can never be too many.  Launch that many back to back, look at the counters once, repeat.
+    // (A launch of the whole-step kernel ends by itself when there is nothing left to do: twice that many may be asked for.)
     int64_t launches = 0;
-    bool have_tokens = false;
+    bool have_tokens = false, stepped = false;
     CU_TRY(cudaEventRecord(e->ev0, e->stream));
     // the first step's plan; every graph launch then ends with the plan of the step after it
-    {
+    if (!whole || max_new == 0) {
         const int64_t before = e->launch_counter;
         enqueue_tail(e, n, k, false, true);
         launches += e->launch_counter - before;
@@ -589,9 +621,17 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         }
         if (left <= 0) break;
         const int batch = (left + k) / (k + 1);
-        rc = launch_steps(e, graph, n, k, batch);
+        if (whole) {
+            const int64_t before = e->launch_counter;
+            rc = enqueue_whole_steps(e, n, k, std::min(left, std::max(kStepsPerLaunch, 2 * batch)), !stepped, true);
+            launches += e->launch_counter - before;
+            e->launch_counter = before;
+        } else {
+            rc = launch_steps(e, graph, n, k, batch);
+            launches += (int64_t)batch * e->launches_per_step;
+        }
         if (rc) return rc;
-        launches += (int64_t)batch * e->launches_per_step;
+        stepped = true;
         // the last look at the state brings the tokens too (a few kilobytes at most: it may be any look)
         const bool with_tokens = (size_t)(y_hi - y_lo) * d.max_batch <= 16384;
         if (with_tokens) { rc = copy_tokens(e, y_lo, y_hi); if (rc) return rc; }
@@ -601,7 +641,7 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         have_tokens = with_tokens;
         if (*e->h_err != kDevErrNone) break;
     }
-    if (launches <= 1) {  // no step was taken
+    if (!stepped) {  // no step was taken
         CU_TRY(cudaEventRecord(e->ev1, e->stream));
         rc = pull_state(e);
         if (rc) return rc;
@@ -681,14 +721,20 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
     if (rc) return rc;
     CU_TRY(cudaStreamSynchronize(e->stream));  // the host arrays may go after this
     cudaGraphExec_t graph = nullptr;
-    rc = get_step_graph(e, 1, 0, &graph);
-    if (rc) return rc;
+    if (!e->step_simt) {
+        rc = get_step_graph(e, 1, 0, &graph);
+        if (rc) return rc;
+    }
     CU_TRY(cudaEventRecord(e->ev0, e->stream));
     const int64_t before = e->launch_counter;
-    enqueue_tail(e, 1, 0, false, true);
-    const int64_t tail_launches = e->launch_counter - before;
+    if (e->step_simt) rc = enqueue_whole_steps(e, 1, 0, n_steps, true, true);
+    else enqueue_tail(e, 1, 0, false, true);
+    int64_t launches = e->launch_counter - before;
     e->launch_counter = before;
-    rc = launch_steps(e, graph, 1, 0, n_steps);
+    if (!e->step_simt) {
+        rc = launch_steps(e, graph, 1, 0, n_steps);
+        launches += (int64_t)n_steps * e->launches_per_step;
+    }
     if (rc) return rc;
     CU_TRY(cudaEventRecord(e->ev1, e->stream));
     rc = pull_state(e);
@@ -706,7 +752,7 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
         T.forced_rows = 0; T.forced_emit = 0; T.trace_step = 0;
         e->state_dirty = true;
     }
-    st.launches = tail_launches + (int64_t)n_steps * e->launches_per_step;
+    st.launches = launches;
     CU_TRY(cudaEventElapsedTime(&st.device_ms, e->ev0, e->ev1));
     if (stats) *stats = st;
     e->last_step_valid = false;

@@ -20,7 +20,7 @@
 // how many rows the step has.  That is what makes a (k+1)-row verification step bit-identical to k+1 one-row steps.
 #include <type_traits>
 
-#include "kernels.h"
+#include "simt_common.cuh"
 
 namespace llma {
 
@@ -28,26 +28,6 @@ constexpr int kWarps = 8;        // warps per CTA
 constexpr int kRB = 16;          // most activation rows per pass over the weights
 constexpr int kKC = 512;         // columns whose weights a warp holds at a time
 constexpr size_t kResidentBytes = 200 * 1024;  // activation rows that fit stay in shared memory whole
-
-// 16 bytes of a weight row as floats
-template <typename T> struct Vec16;
-template <> struct Vec16<float> {
-    static constexpr int N = 4;
-    __device__ static void widen(const uint4& t, float (&v)[4]) {
-        v[0] = __uint_as_float(t.x); v[1] = __uint_as_float(t.y); v[2] = __uint_as_float(t.z); v[3] = __uint_as_float(t.w);
-    }
-};
-template <> struct Vec16<__nv_bfloat16> {
-    static constexpr int N = 8;
-    __device__ static void widen(const uint4& t, float (&v)[8]) {
-        const uint32_t w[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[2 * i] = __uint_as_float(w[i] << 16);
-            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-        }
-    }
-};
 
 // The sums of 32 (feature, row) pairs, one per lane: value f * 16 + r of every lane is added over the lanes and
 // ends in lane f * 16 + r.  The same tree for every value.
