@@ -323,17 +323,17 @@ int llma_gemm_rows32_bf16(const void *W, const void *a, float *out, int32_t n_ou
  * no cudaMalloc, cudaFree or any other allocating routine.
  *
  * Arguments, layouts and results are exactly those of llma_gemm_rows32_bf16 (W, a, out are
- * caller-owned device buffers).  The partial tiles handed between CTAs and the error word live in a fixed
+ * caller-owned device buffers).  The partial tiles handed between CTAs live in a fixed
  * array of about 2.5 MiB that is part of the library image: every GPU that loads the library holds it until
  * the process exits.  Limits: n_out <= 262144 and k_in <= 16384; larger sizes return LLMA_ERR_CAPACITY
  * and do nothing.
  *
  * The first call on a device resolves the array's device address (with the caller's current
- * device) and opts the kernel into its shared-memory size.  All calls on a device share the array
- * and it keeps the previous call's contents: the call itself puts the hand-over slots into their
- * empty state and clears the error word, but two calls that overlap on the GPU (different streams,
- * or different threads) race on it and give wrong results -- serialise them.  The call is
- * synchronous: it waits for the kernel and reads its error word back before it returns.
+ * device), opts the kernel into its shared-memory size and pins a page of the library's own host memory for the
+ * error words.  All calls on a device share the array and it keeps the previous call's contents: a call leaves the
+ * hand-over slots empty, and empties them first if the call before did not end well, but two calls that overlap on
+ * the GPU (different streams, or different threads) race on it and give wrong results -- serialise them.  The call is
+ * synchronous: it waits for the kernel and looks at its error word before it returns.
  * Errors: NULL, ARG, CAPACITY, CONFIG (not an sm_100 device), CUDA, DEVICE_TIMEOUT.
  */
 int llma_gemm_rows32_bf16_noalloc(const void *W, const void *a, float *out, int32_t n_out, int32_t k_in,

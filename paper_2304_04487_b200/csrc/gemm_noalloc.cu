@@ -1,6 +1,5 @@
 // llma_gemm_rows32_bf16_noalloc: the stand-alone projection GEMM for callers that must not
-// allocate.  Its partial tiles (handed between CTAs) and error word live in one file-scope __device__ array
-// instead of cudaMalloc'ed memory.
+// allocate.  Its partial tiles (handed between CTAs) live in one file-scope __device__ array instead of cudaMalloc'ed memory.
 #include <mutex>
 
 #include "engine.h"
@@ -21,14 +20,22 @@ constexpr int kMaxK = 16384;
 constexpr size_t kWsBytes = gemm_ws_bytes(kMaxGrid);  // 2,621,440
 
 // Every GPU that loads this library holds this array until the process exits.  In host code the name below is only a
-// handle for cudaGetSymbolAddress, never a device address.  The error word lies before the slots, so that one
-// memset reaches it and the slots of the grid in use.
-constexpr size_t kErrBytes = 256;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kErrBytes + kWsBytes];
+// handle for cudaGetSymbolAddress, never a device address.
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kWsBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-unsigned char* g_scratch_ptr[kMaxDevices] = {nullptr};
+struct Scratch {
+    float* ws = nullptr;   // device address of the array
+    bool clean = false;    // every hand-over word is empty: the calls before have ended well, one at a time
+    int calls = 0;         // under way now
+    bool mixed = false;    // ... more than one at some time: what they leave is anyone's guess
+};
+Scratch g_scratch[kMaxDevices];
+// Error words, one per device, that the kernel writes when a wait runs out: host memory of the library's own, pinned by the first
+// call, so that a call reads them without a copy.  A page to themselves, since pages are what is pinned.
+alignas(4096) int32_t g_err[4096 / sizeof(int32_t)];
+int32_t* g_err_dev = nullptr;  // ... as the devices see them
 
 }  // namespace
 
@@ -41,29 +48,53 @@ extern "C" int llma_gemm_rows32_bf16_noalloc(const void* W, const void* a, float
     int dev = 0, sms = 0;
     int rc = gemm_device(&dev, &sms);
     if (rc) return rc;
-    unsigned char* base = nullptr;
+    Scratch& sc = g_scratch[dev];
+    float* ws = nullptr;
+    int32_t* err_dev = nullptr;
+    bool clean = false;
     {
-        // one-time set-up per device, with that device current: resolve the array's device address
+        // set-up, with the device current: the array's address and the pinned words
         std::lock_guard<std::mutex> lock(g_mu);
-        if (!g_scratch_ptr[dev]) {
-            unsigned char* p = nullptr;
-            CU_TRY(cudaGetSymbolAddress((void**)&p, g_noalloc_scratch));
-            g_scratch_ptr[dev] = p;
+        if (!sc.ws) {
+            void* p = nullptr;
+            CU_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch));
+            if (!g_err_dev) {
+                void* q = nullptr;
+                CU_TRY(cudaHostRegister(g_err, sizeof(g_err), cudaHostRegisterPortable | cudaHostRegisterMapped));
+                CU_TRY(cudaHostGetDevicePointer(&q, g_err, 0));
+                g_err_dev = static_cast<int32_t*>(q);
+            }
+            sc.ws = static_cast<float*>(p);
         }
-        base = g_scratch_ptr[dev];
+        ws = sc.ws;
+        err_dev = g_err_dev + dev;
+        clean = sc.clean && sc.calls == 0;
+        sc.mixed = sc.mixed || sc.calls > 0;
+        sc.calls += 1;
+        sc.clean = false;
     }
-    int32_t* err_dev = reinterpret_cast<int32_t*>(base);
-    float* ws = reinterpret_cast<float*>(base + kErrBytes);
+    struct Leave {  // the call is over, by whichever return
+        Scratch& sc;
+        bool well = false;
+        ~Leave() {
+            std::lock_guard<std::mutex> lock(g_mu);
+            if (--sc.calls > 0) return;
+            sc.clean = well && !sc.mixed;
+            sc.mixed = false;
+        }
+    } leave{sc};
     cudaStream_t st = (cudaStream_t)cuda_stream;
     int grid = gemm_grid_for((int64_t)n_tiles * (k_in / 64), sms);
     if (grid > kMaxGrid) grid = kMaxGrid;
-    // the array keeps the previous call's contents, which may have been cut short: one memset empties the hand-over
-    // slots (all-ones words) and puts the error word to all-ones, which no error code is
-    CU_TRY(cudaMemsetAsync(base, 0xFF, kErrBytes + gemm_ws_bytes(grid), st));
+    // A call leaves the hand-over slots empty (all-ones words), as it needs them.  After one that did not end well, and for the first, all of them
+    // are emptied: 2.6 MB, which with the error word copied back was a quarter of a call (22016 x 4096: 61.5 -> 49.0 us).
+    volatile int32_t* err = g_err + dev;
+    if (!clean) CU_TRY(cudaMemsetAsync(ws, 0xFF, kWsBytes, st));
+    *err = kDevErrNone;
     rc = gemm_rows32_launch(W, a, out, n_out, k_in, ws, err_dev, grid, st);
-    if (rc) return rc;
-    int32_t err = 0;
-    CU_TRY(cudaMemcpyAsync(&err, err_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    if (rc && rc != LLMA_ERR_ARG) return rc;
     CU_TRY(cudaStreamSynchronize(st));
-    return err == -1 ? LLMA_OK : LLMA_ERR_DEVICE_TIMEOUT;
+    if (rc == LLMA_OK && *err != kDevErrNone) return LLMA_ERR_DEVICE_TIMEOUT;
+    leave.well = true;
+    return rc;
 }

@@ -47,6 +47,23 @@ def test_noalloc_matches_allocating_entry_point_twice():
     assert free_after == free_before
 
 
+@pytest.mark.parametrize("sizes", [[(4096, 4096), (128, 64), (4096, 4096), (1000, 1024)]])   # grids of 148, 1, 148 and 16 CTAs in turn
+def test_noalloc_scratch_serves_every_grid(sizes):
+    """The hand-over slots are emptied once and then left empty by every call, whatever part of them it uses; a refused call
+    in between changes nothing."""
+    import torch
+    from paper_2304_04487_b200 import LlmaError, llma_gemm_rows32_bf16, llma_gemm_rows32_bf16_noalloc
+    for i, (n_out, k_in) in enumerate(sizes):
+        W, a = _rand_bf16((n_out, k_in), 0.05, i), _rand_bf16((32, k_in), 1.0, 50 + i)
+        want, got = torch.empty((32, n_out), device="cuda"), torch.full((32, n_out), float("nan"), device="cuda")
+        llma_gemm_rows32_bf16(W, a, want)
+        llma_gemm_rows32_bf16_noalloc(W, a, got)
+        assert torch.equal(got, want), (n_out, k_in)
+        flat = torch.zeros(n_out * k_in + 8, dtype=torch.bfloat16, device="cuda")
+        with pytest.raises(LlmaError):
+            llma_gemm_rows32_bf16_noalloc(flat[1:1 + n_out * k_in].view(n_out, k_in), a, got)
+
+
 def test_noalloc_matches_oracle_directly():
     """The same entry point against the CPU oracle's matrix-vector product, with no other entry point in between."""
     import torch
