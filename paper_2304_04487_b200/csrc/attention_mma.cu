@@ -355,15 +355,17 @@ __global__ void __launch_bounds__(128, 3) attention_long_kernel(const AttnArgs a
     volatile uint32_t* flag = reinterpret_cast<volatile uint32_t*>(bar + 2);
     const uint32_t bar_u = smem_u32(bar), bar_v = bar_u + 8;  // K tile, V tile
 
+    // (rows that come through once per step, 67 MB and more a layer: see l2_evict_first; sixteen 7B-shaped sequences of 4096 positions 33.6 -> 32.0 ms,
+    // where one sequence's rows in attention_mma_kernel are better left alone, 64.2 against 64.7)
     auto fetch_k = [&](int t) {  // one thread
         const int32_t row0 = (int32_t)kv_row_index(d, a.layer, seq, head, c0 + t * kAttnChunk);
         mbar_arrive_expect_tx(bar_u, L::kTileBytes);
-        for (int b = 0; b < L::kBoxes; ++b) tma_load_2d(base + L::offK + b * L::kBoxBytes, &map_k, bar_u, b * 64, row0);
+        for (int b = 0; b < L::kBoxes; ++b) tma_load_2d(base + L::offK + b * L::kBoxBytes, &map_k, bar_u, b * 64, row0, l2_evict_first());
     };
     auto fetch_v = [&](int t) {
         const int32_t row0 = (int32_t)kv_row_index(d, a.layer, seq, head, c0 + t * kAttnChunk);
         mbar_arrive_expect_tx(bar_v, L::kTileBytes);
-        for (int b = 0; b < L::kBoxes; ++b) tma_load_2d(base + L::offV + b * L::kBoxBytes, &map_v, bar_v, b * 64, row0);
+        for (int b = 0; b < L::kBoxes; ++b) tma_load_2d(base + L::offV + b * L::kBoxBytes, &map_v, bar_v, b * 64, row0, l2_evict_first());
     };
     // the first tile may be requested before the QKV projection has finished if it lies wholly below the committed length
     const int kv_len = __ldcg(&a.seq_state[seq].kv_len);

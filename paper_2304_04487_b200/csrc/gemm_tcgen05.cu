@@ -107,18 +107,21 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
     if (warp == 4) {
         // ------------------------------- producer ---------------------------------------------
         if (elect_one()) {
+            const uint64_t policy = MODE == kGemmStore ? 0 : l2_evict_first();
             auto load_a = [&](int tile, int c, int s) {
                 const uint32_t dstA = sA + s * kABytes;
                 // chunks 2c and 2c+1 of the tile in one copy (a chunk past the matrix arrives as zeros)
                 if (MODE == kGemmSwiGLU) {  // 64 rows of each of the two matrices per chunk
-                    tma_load_4d(dstA, &map_a0, full_bar(s), 0, tile * 64, 0, c * KC);
+                    tma_load_4d(dstA, &map_a0, full_bar(s), 0, tile * 64, 0, c * KC, policy);
                 } else {
                     const CUtensorMap* mp = &map_a0;
                     if (MODE == kGemmQKV) {
                         if (tile >= 2 * g.tiles_per_map) { mp = &map_a2; tile -= 2 * g.tiles_per_map; }
                         else if (tile >= g.tiles_per_map) { mp = &map_a1; tile -= g.tiles_per_map; }
                     }
-                    tma_load_3d(dstA, mp, full_bar(s), 0, tile * 128, c * KC);
+                    // (the matrix of a stand-alone product may be multiplied again at once: 27.7 us a call against 28.8 with the hint)
+                    if (MODE == kGemmStore) tma_load_3d(dstA, mp, full_bar(s), 0, tile * 128, c * KC);
+                    else tma_load_3d(dstA, mp, full_bar(s), 0, tile * 128, c * KC, policy);
                 }
             };
             // weights are written by no kernel of the step: the whole range streams without waiting for

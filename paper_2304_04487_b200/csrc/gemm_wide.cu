@@ -115,6 +115,7 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
     if (warp == 4) {
         // ------------------------------- weight producer ------------------------------------------
         if (elect_one()) {
+            const uint64_t policy = l2_evict_first();
             int it = 0;
             int tile = tile0, c = c_beg;
             int m = 0, rt = tile;  // matrix and tile inside it
@@ -128,11 +129,11 @@ gemm_wide_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ CUt
                 mbar_arrive_expect_tx(full_bar(s), kGemmABytes);
                 const uint32_t dstA = sA + (uint32_t)s * stage_bytes;
                 if (MODE == kGemmSwiGLU) {
-                    tma_load_2d(dstA, &map_a0, full_bar(s), c * 64, tile * 64);
-                    tma_load_2d(dstA + kGemmABytes / 2, &map_a1, full_bar(s), c * 64, tile * 64);
+                    tma_load_2d(dstA, &map_a0, full_bar(s), c * 64, tile * 64, policy);
+                    tma_load_2d(dstA + kGemmABytes / 2, &map_a1, full_bar(s), c * 64, tile * 64, policy);
                 } else {
                     const CUtensorMap* mp = m == 0 ? &map_a0 : (m == 1 ? &map_a1 : &map_a2);
-                    tma_load_2d(dstA, mp, full_bar(s), c * 64, rt * 128);
+                    tma_load_2d(dstA, mp, full_bar(s), c * 64, rt * 128, policy);
                 }
                 if (++c == C) { c = 0; ++tile; if (++rt == g.tiles_per_map) { rt = 0; ++m; } }
                 if (++s == S) { s = 0; ph ^= 1u; }

@@ -91,6 +91,35 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
 }
+// The same for data that comes through once per step, above all the weights: their lines are the first to leave L2.  A layer of the 7B shape
+// streams 400 MB through 126 MB; without the hint everything small that it needs again -- code, activations, partial tiles, row
+// descriptors -- has left by the next layer, and the ends of every launch wait for DRAM (us per pass, one 7B-shaped sequence: first MMA of
+// QKV 2.2 -> 1.8 after its predecessor, last CTA 17.3 -> 16.4; decodes: 7B one row 66.9 -> 64.2 ms, up to nine 91.8 -> 88.1, 13B up to
+// seventeen 105.9 -> 100.4, four 7B-shaped sequences 14.3 -> 13.3).  Decoders whose weights fit L2 do not notice.
+__device__ __forceinline__ uint64_t l2_evict_first() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t x, int32_t y, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t x, int32_t y, int32_t z, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t x, int32_t y, int32_t z,
+                                            int32_t w, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy)
+        : "memory");
+}
 // A load that is really performed every time it is executed, at GPU scope (for polling memory that
 // another CTA writes): the compiler may neither hoist it out of a loop nor reuse an earlier value.
 __device__ __forceinline__ float4 ld_poll_f4(const float4* p) {
