@@ -59,7 +59,7 @@ static void free_engine(llma_engine* e) {
     cudaFree(e->rope_cos); cudaFree(e->rope_sin); cudaFree(e->kcache); cudaFree(e->vcache);
     cudaFree(e->attn_ws_o); cudaFree(e->attn_ws_ml); cudaFree(e->trace); cudaFree(e->target);
     cudaFree(e->gemm_ws); cudaFree(e->stamps); cudaFree(e->gemm_ws_wide); cudaFree(e->gemm_flags); cudaFree(e->part_max); cudaFree(e->part_idx); cudaFree(e->norm_ss);
-    cudaFree(e->p_tok); cudaFree(e->step_ops); cudaFree(e->grid_barrier); cudaFree(e->ll_words);
+    cudaFree(e->p_tok); cudaFree(e->ll_words);
     free_prompt_buffers(e);
     if (e->h_block) cudaFreeHost(e->h_block);
     for (int i = 0; i < 2; ++i)
@@ -85,7 +85,7 @@ static cudaError_t alloc_prompt_buffers(llma_engine* e) {
     return r;
 }
 
-// Whole decoding steps of the CUDA-core path in one launch, where the rows of a pass fit shared memory
+// Whole decoding steps on the CUDA cores in one launch, where the rows of a pass fit shared memory
 static cudaError_t init_whole_steps(llma_engine* e) {
     const ModelDims& d = e->dims;
     int coop = 0;
@@ -104,15 +104,17 @@ static cudaError_t init_whole_steps(llma_engine* e) {
         ops.push_back({e->w_down[l], nullptr, nullptr, nullptr});
     }
     ops.push_back({e->lm_head, nullptr, nullptr, e->final_norm});
-    if ((r = dalloc(&e->step_ops, ops.size(), false)) != cudaSuccess) return r;
-    if ((r = cudaMemcpy(e->step_ops, ops.data(), ops.size() * sizeof(SimtOp), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
-    if ((r = dalloc(&e->grid_barrier, 1)) != cudaSuccess) return r;
     const size_t rc = (size_t)e->row_cap, parts = 2 * (size_t)e->num_sms * rc;
     e->ll_count = rc * (d.d_model + 4 * (size_t)d.hd_total + d.d_ffn) + parts + simt_rows_words(e->row_cap);
-    if ((r = dalloc(&e->ll_words, e->ll_count)) != cudaSuccess) return r;
+    // one block: the words, the barrier's, the ops
+    const size_t words = e->ll_count + 1 + (ops.size() * sizeof(SimtOp) + 7) / 8;
+    if ((r = dalloc(&e->ll_words, words)) != cudaSuccess) return r;
+    e->grid_barrier = reinterpret_cast<uint32_t*>(e->ll_words + e->ll_count);
+    SimtOp* step_ops = reinterpret_cast<SimtOp*>(e->ll_words + e->ll_count + 1);
+    if ((r = cudaMemcpy(step_ops, ops.data(), ops.size() * sizeof(SimtOp), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
     s.ll_x = e->ll_words; s.ll_qkv = s.ll_x + rc * d.d_model; s.ll_attn = s.ll_qkv + rc * 3 * d.hd_total;
     s.ll_h = s.ll_attn + rc * d.hd_total; s.ll_part = s.ll_h + rc * d.d_ffn; s.ll_rows = s.ll_part + parts;
-    s.dims = d; s.ops = e->step_ops; s.emb = e->tok_emb; s.rows = e->rows;
+    s.dims = d; s.ops = step_ops; s.emb = e->tok_emb; s.rows = e->rows;
     s.x = e->x; s.qkv = e->qkv; s.attn = (float*)e->attn; s.h = (float*)e->h; s.logits = e->cfg.keep_logits ? e->logits : nullptr;
     s.kcache = e->kcache; s.vcache = e->vcache; s.rope_cos = e->rope_cos; s.rope_sin = e->rope_sin;
     s.barrier = e->grid_barrier; s.dev_err = e->dev_err;
@@ -345,6 +347,15 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
             if (e->prompt_pairs < 1) { free_engine(e); return LLMA_ERR_CONFIG; }
         }
     }
+    // Decoding steps of narrow decoders run whole on the CUDA cores: at these widths a step costs the ends of its launches, not its
+    // weights.  The line lies where the two cost the same.  us per decode, launches of tensor-core kernels -> whole steps: width 256, two
+    // layers, up to 16 rows at 700 positions 1202 -> 844, four sequences 1834 -> 1359; width 512, three layers, up to six rows, a call per
+    // step 1536 -> 1335, up to 16 rows at 700 positions 1649 -> 1404, two sequences 1837 -> 1779, four 2409 -> 2438; width 1024, two
+    // layers, up to nine rows at 600 positions 1987 -> 1965, up to thirteen at 2000 positions 1993 -> 2672 (a row and head is one CTA's
+    // work here, 0.6 us per 64 positions).  All rows in one pass; an engine asked for the tensor cores keeps to them.
+    if (e->gemm_impl == LLMA_GEMM_TCGEN05 && cfg->gemm_impl == LLMA_GEMM_AUTO && e->decode_rows <= 16 && d.d_model <= 512 &&
+        d.d_model * d.max_batch <= 1024 && d.max_seq <= 768)
+        CREATE_TRY(init_whole_steps(e));
     {
         // page-locked memory in one piece: every such allocation costs about a millisecond
         size_t total = 0;

@@ -78,14 +78,14 @@ struct llma_engine {
     int attn_tiles = 1;             // 128-position tiles per attention CTA in decoding steps (a function of the capacity only)
     float *attn_ws_o = nullptr, *attn_ws_ml = nullptr;
 
-    // whole steps in one cooperative launch: CUDA-core path (step_simt.cu)
+    // whole steps in one cooperative launch (step_simt.cu): CUDA-core path, and narrow decoders of the tensor-core path
     bool step_simt = false;
+    bool plain_acts = false;        // attn and h hold fp32 rows (of a whole step), whatever the path
     llma::SimtStep simt{};          // everything that does not change from launch to launch
     size_t simt_smem = 0;
-    llma::SimtOp* step_ops = nullptr;
-    uint32_t* grid_barrier = nullptr;
-    unsigned long long* ll_words = nullptr;   // activations on their way from CTA to CTA
+    unsigned long long* ll_words = nullptr;   // activations on their way from CTA to CTA; behind them the barrier's word and the ops
     size_t ll_count = 0;
+    uint32_t* grid_barrier = nullptr;
     uint32_t ll_epoch = 1;                    // first number of the next launch
 
     // replay of a given step sequence (llma_generate_forced)

@@ -185,7 +185,7 @@ extern "C" int llma_debug_buffer(llma_engine* e, int32_t which, float* out, int6
         return LLMA_OK;
     }
     const void* src = which == 2 ? e->attn : e->h;
-    if (e->gemm_impl != LLMA_GEMM_TCGEN05) {  // fp32 [32][K]
+    if (e->gemm_impl != LLMA_GEMM_TCGEN05 || e->plain_acts) {  // fp32 [32][K]
         CU_TRY(cudaMemcpy(out, src, (size_t)count * sizeof(float), cudaMemcpyDeviceToHost));
         return LLMA_OK;
     }

@@ -194,6 +194,7 @@ static void enqueue_tail(llma_engine* e, int n, int k, bool accept, bool plan) {
 // llma_generate's graph) the plan of the next step in the same launch.
 static void enqueue_step_body(llma_engine* e, int n, int k, bool plan_next) {
     e->cur_rows = e->decode_rows;
+    e->plain_acts = false;
     e->launch_seq = 0;
     enqueue_embed(e);
     mark(e, LLMA_K_EMBED);
@@ -206,6 +207,7 @@ static void enqueue_step_body(llma_engine* e, int n, int k, bool plan_next) {
 // the first one (otherwise the launch before has planned it); plan_last: plan the step after the last one.
 static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps, bool plan_first, bool plan_last) {
     SimtStep s = e->simt;
+    e->plain_acts = true;
     s.tail = tail_args(e, n, k);
     const uint32_t per_step = simt_epochs(e->dims);
     for (; steps > 0; steps -= kStepsPerLaunch, plan_first = false) {

@@ -39,3 +39,27 @@ def test_generate_equals_single_steps(d, heads, hd, ffn, vocab, k, B, N):
             got[s] += t
     assert [g[:N] for g in got] == greedy
     eng.llma_destroy()
+
+
+@pytest.mark.parametrize("impl", [0, 2])   # whole steps (narrow, few rows, short contexts), and the launches that they stand in for
+@pytest.mark.parametrize("name,k", [("tiny-bf16", 8), ("small-bf16", 15)])
+def test_narrow_decoders_both_ways(name, k, impl):
+    from oracle import model as OM
+    from parity import step_parity
+    from paper_2304_04487_b200 import Engine
+    from workloads import SHAPES, build_reference
+    shape = SHAPES[name]
+    w = make_weights(shape, seed=0)
+    P, N = 290, 24
+    prompt = make_prompt(P, shape.vocab, seed=2)
+    eng = Engine(shape, w, max_seq=P + N + 40, max_ref=200, max_k=k, gemm_impl=impl, keep_logits=True)
+    assert eng.llma_gemm_impl() == 2
+    eng.llma_prefill(0, prompt)
+    (y,), st = eng.llma_generate(N, 1, 0)
+    assert st.launches == (1 if impl == 0 else 1 + N * (3 + 6 * shape.n_layers))
+    ref, offs, _ = build_reference(y, [60, 60, 40], 0.7, shape.vocab, seed=1)
+    rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=P + N + 40), prompt, ref, offs, 1, k, N, "bf16")
+    assert rep.max_logit_err <= 2e-2 and rep.near_ties <= 3 and rep.trigger_steps > 0
+    prof = eng.llma_profile_steps(1, k, 2)                  # launch by launch, on the same engine
+    assert prof["_total"]["launches_per_step"] == 4 + 5 * shape.n_layers   # (the two attention kernels count as one)
+    eng.llma_destroy()
