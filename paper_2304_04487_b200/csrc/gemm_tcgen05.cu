@@ -26,6 +26,8 @@
 // issuing work, lets its outstanding copies land, frees TMEM and returns.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "gemm_epilogue.cuh"
 #include "gemm_tcgen05.cuh"
 #include "ptx_sm100.cuh"
@@ -451,52 +453,60 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
 #pragma unroll 1
                 while (begin_of(b_last + 1) < t_hi) ++b_last;
                 const unsigned long long give_up = globaltimer_ns() + 2000000000ull;
-                constexpr int kBatch = NR == 32 ? 1 : 2;  // partials requested together (registers)
+                // kQ groups of four rows, the partials of kBatch CTAs requested together: a batch costs a trip to L2 at least.  With up to
+                // four rows all partials that a tile usually has are one batch (us per decode, two CTAs a batch -> six: 7B shape, one row,
+                // 65030 -> 64320, up to nine 88260 -> 87060); more than two at a time of all rows gain nothing (87130) and one of 32 rows
+                // less (13B shape, up to seventeen rows, 104460 -> 102700 with it, 102340 with two).
+                auto collect = [&](auto q_tag, auto batch_tag) {
+                    constexpr int kQ = decltype(q_tag)::value, kBatch = decltype(batch_tag)::value;
 #pragma unroll 1
-                for (int bb = b + 1; bb <= b_last; bb += kBatch) {  // ascending k: a fixed summation order
-                    float4 p[kBatch][NR / 4];
-                    bool valid;
-                    do {
-                        valid = true;
+                    for (int bb = b + 1; bb <= b_last; bb += kBatch) {  // ascending k: a fixed summation order
+                        float4 p[kBatch][kQ];
+                        bool valid;
+                        do {
+                            valid = true;
 #pragma unroll
-                        for (int u = 0; u < kBatch; ++u) {
-                            if (bb + u <= b_last) {
-                                const float4* src = ws_slot(g.ws, NR / 4, bb + u, row);
+                            for (int u = 0; u < kBatch; ++u) {
+                                if (bb + u <= b_last) {
+                                    const float4* src = ws_slot(g.ws, NR / 4, bb + u, row);
 #pragma unroll
-                                for (int q = 0; q < NR / 4; ++q)
-                                    if (4 * q < rows_used) p[u][q] = ld_poll_f4(src + q * 128);
+                                    for (int q = 0; q < kQ; ++q)
+                                        if (kQ == 1 || 4 * q < rows_used) p[u][q] = ld_poll_f4(src + q * 128);
+                                }
                             }
-                        }
+#pragma unroll
+                            for (int u = 0; u < kBatch; ++u) {
+                                if (bb + u <= b_last) {
+#pragma unroll
+                                    for (int q = 0; q < kQ; ++q) {
+                                        if (kQ == 1 || 4 * q < rows_used) {
+                                            valid = valid && __float_as_uint(p[u][q].x) != kEmpty && __float_as_uint(p[u][q].y) != kEmpty &&
+                                                    __float_as_uint(p[u][q].z) != kEmpty && __float_as_uint(p[u][q].w) != kEmpty;
+                                        }
+                                    }
+                                }
+                            }
+                            if (!valid && globaltimer_ns() > give_up) { atomicExch(g.dev_err, kDevErrTimeout); break; }
+                        } while (!valid);
+                        const float e = __uint_as_float(kEmpty);
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
                             if (bb + u <= b_last) {
+                                float4* src = ws_slot(g.ws, NR / 4, bb + u, row);
 #pragma unroll
-                                for (int q = 0; q < NR / 4; ++q) {
-                                    if (4 * q < rows_used) {
-                                        valid = valid && __float_as_uint(p[u][q].x) != kEmpty && __float_as_uint(p[u][q].y) != kEmpty &&
-                                                __float_as_uint(p[u][q].z) != kEmpty && __float_as_uint(p[u][q].w) != kEmpty;
+                                for (int q = 0; q < kQ; ++q) {
+                                    if (kQ == 1 || 4 * q < rows_used) {
+                                        src[q * 128] = make_float4(e, e, e, e);  // empty again for the next projection
+                                        acc[4 * q] += p[u][q].x; acc[4 * q + 1] += p[u][q].y;
+                                        acc[4 * q + 2] += p[u][q].z; acc[4 * q + 3] += p[u][q].w;
                                     }
                                 }
                             }
                         }
-                        if (!valid && globaltimer_ns() > give_up) { atomicExch(g.dev_err, kDevErrTimeout); break; }
-                    } while (!valid);
-                    const float e = __uint_as_float(kEmpty);
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        if (bb + u <= b_last) {
-                            float4* src = ws_slot(g.ws, NR / 4, bb + u, row);
-#pragma unroll
-                            for (int q = 0; q < NR / 4; ++q) {
-                                if (4 * q < rows_used) {
-                                    src[q * 128] = make_float4(e, e, e, e);  // empty again for the next projection
-                                    acc[4 * q] += p[u][q].x; acc[4 * q + 1] += p[u][q].y;
-                                    acc[4 * q + 2] += p[u][q].z; acc[4 * q + 3] += p[u][q].w;
-                                }
-                            }
-                        }
                     }
-                }
+                };
+                if (rows_used <= 4) collect(std::integral_constant<int, 1>{}, std::integral_constant<int, 6>{});
+                else collect(std::integral_constant<int, NR / 4>{}, std::integral_constant<int, 2>{});
             }
             if (threadIdx.x == 0 && live) LLMA_STAMP(stp, 6);  // partials summed: the tile's epilogue begins
             finish_tile(tile, acc, xpre, live);
