@@ -19,8 +19,8 @@
 // take a first turn that loads and stores nothing while they have nothing else to do, which brings their code in.
 // us per pass, before -> after: three layers of width 512 at up to six rows 116 -> 110 for the counting and 118 -> 116 for
 // the turns; 7B shape, one row, 2755 -> 2715 for the turns; no difference at nine rows.  More code in the same place costs
-// more than it hides: four rows abreast in the epilogues, warmed up the same way, 2715 -> 2766; the partials of four CTAs
-// requested together, and before the accumulator is ready, 2685 -> 2805.
+// more than it hides: four rows abreast in the epilogues, warmed up the same way, 2715 -> 2766; the first partials
+// requested before the accumulator is ready, four CTAs' at a time, 2685 -> 2805.
 //
 // Every wait is bounded: when one runs out the kernel raises the device error word, stops
 // issuing work, lets its outstanding copies land, frees TMEM and returns.

@@ -1,5 +1,5 @@
-// Whole decoding steps of the CUDA-core path (fp32 models, and the cross-check of the tensor-core path) in one cooperative
-// launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
+// Whole decoding steps on the CUDA cores (fp32 models, the cross-check of the tensor-core path, and narrow bf16 decoders: the rule and
+// what it measured are in engine.cu) in one cooperative launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
 //
 // At the widths this path serves a step is a chain of short phases and costs their latency.  As launches of their own
 // (kernels_simt.cu, attention_simt.cu) a phase is released about 1 us after its predecessor has ended, fetches its rows, and runs
@@ -22,8 +22,8 @@
 // 42 -> 34 us per step of width 256 for this alone), one and two rows have code of their own, and nothing is spilled: local memory does not
 // fit what 226 KB of shared memory leave of L1, and a reload comes from L2 or further (2 us at the end of the attention phase of
 // width 1024).  Feeders give up registers for the warps that multiply for that reason.
-// us per decode, as launches -> here: two fp32 layers of width 256, 64 tokens, up to five rows 2522 -> 1446; of width 1024, up to nine
-// rows 2673 -> 1935 (its weights, 135 MB a step, take 450); up to 76 rows, in five passes over the weights, 3435 -> 3430.
+// us per decode, as launches -> here: two fp32 layers of width 256, 64 tokens, up to five rows 2483 -> 1443; of width 1024, up to nine
+// rows 2709 -> 1863 (its weights, 135 MB a step, take 450); up to 76 rows, in five passes over the weights, 3435 -> 3430.
 //
 // Every sum is a fixed sequence of operations that depends on its own row's data and on the shapes only, never on how many rows the
 // step has.
