@@ -505,8 +505,9 @@ gemm_ws_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap map_a0, con
                         }
                     }
                 };
-                if (rows_used <= 4) collect(std::integral_constant<int, 1>{}, std::integral_constant<int, 6>{});
-                else collect(std::integral_constant<int, NR / 4>{}, std::integral_constant<int, 2>{});
+                // (a step without rows, after the last sequence has met its EOS: nothing has been handed over and nothing comes)
+                if (rows_used > 4) collect(std::integral_constant<int, NR / 4>{}, std::integral_constant<int, 2>{});
+                else if (rows_used > 0) collect(std::integral_constant<int, 1>{}, std::integral_constant<int, 6>{});
             }
             if (threadIdx.x == 0 && live) LLMA_STAMP(stp, 6);  // partials summed: the tile's epilogue begins
             finish_tile(tile, acc, xpre, live);
