@@ -368,10 +368,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
     __shared__ StepRows R;
     __shared__ float s_rs[kSR];                  // RMSNorm scale of a row
     __shared__ int s_fail, s_stop;               // a wait ran out; the feeders may go
-    __shared__ int s_steps, s_passes;            // steps begun, passes over the weights in the last of them
+    __shared__ int s_steps, s_passes[2];         // steps begun, passes over the weights in the last two of them
     __shared__ uint64_t s_bar[2][kSW][kRing];    // a place of a warp's weight ring is full, is empty
     __shared__ float2 s_part[2][kSW][4][kSR];    // a warp's sums of the two features of its four pairs, rounds in turn
-    if (threadIdx.x == 0) { s_fail = 0; s_stop = 0; s_steps = 0; s_passes = 1; }
+    if (threadIdx.x == 0) { s_fail = 0; s_stop = 0; s_steps = 0; }
     if (threadIdx.x < kSW * kRing) {
         mbar_init(smem_u32(&s_bar[0][0][0]) + 8 * threadIdx.x, 32);
         mbar_init(smem_u32(&s_bar[1][0][0]) + 8 * threadIdx.x, 1);
@@ -452,15 +452,16 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         uint32_t phases = (1u << kRing) - 1u;  // of the places' empty barriers
         UnitRows u = {nullptr, nullptr, 0, 0};
         bool find = true, any = true;  // the unit's rows have to be found; the warp has something to multiply at all
-        volatile int *stop = &s_stop, *steps = &s_steps, *passes = &s_passes;
+        volatile int *stop = &s_stop, *steps = &s_steps, *passes = s_passes;
         while (!*stop) {
             bool ready = any;
             if (any && unit >= units) {  // done with a pass over a projection, or not begun
-                // (how many passes a step has is known once it has begun)
+                // (how many passes a step has is known once it has begun, and is read of the step that is being fed: the next one may
+                // have begun meanwhile, the one after it not before this warp's part of the next one has been fed)
                 if (op < 0 || a.passes == 1 || *steps > step) {
                     find = true;
                     unit = (mine >> lg) * G + cta;
-                    if (op < 0 || ++pass_no >= (a.passes == 1 ? 1 : *passes)) {  // the next projection that has pieces for the warp
+                    if (op < 0 || ++pass_no >= (a.passes == 1 ? 1 : passes[step & 1])) {  // the next projection that has pieces for the warp
                         int left = n_ops + 1;
                         do {
                             if (++op == n_ops) { op = 0; ++step; }
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         if (tid == 0 && a.passes > 1) {
             int n = 1;
             for (int r = pass; r < rows_used; r += pass) ++n;
-            *(volatile int*)&s_passes = n;
+            *(volatile int*)&s_passes[step & 1] = n;
             __threadfence_block();
             *(volatile int*)&s_steps = step + 1;
         }

@@ -63,3 +63,33 @@ def test_narrow_decoders_both_ways(name, k, impl):
     prof = eng.llma_profile_steps(1, k, 2)                  # launch by launch, on the same engine
     assert prof["_total"]["launches_per_step"] == 4 + 5 * shape.n_layers   # (the two attention kernels count as one)
     eng.llma_destroy()
+
+
+def test_passes_change_from_step_to_step():
+    """Steps of one, two and three passes over the weights in turn, in one launch: the weights that are on their way into a step's ring
+    are those of its own passes."""
+    from paper_2304_04487_b200 import Engine
+    B, k, N = 4, 9, 120                       # 4 to 40 rows
+    shape = ModelShape("passes", 2, 128, 2, 64, 384, 515, "fp32")
+    eng = Engine(shape, make_weights(shape, seed=0, std=0.05), max_seq=40 + N, max_ref=2 * N, max_k=k, max_batch=B, keep_logits=True)
+    for s in range(B):
+        eng.llma_prefill(s, make_prompt(20 + s, shape.vocab, seed=70 + s))
+    rng = np.random.default_rng(3)
+    y = [int(t) for t in rng.integers(0, shape.vocab, N)]
+    eng.llma_generate_forced(-1, [(1, 1)] * N, y)   # four rows a step
+    eng.llma_step(1, 0)
+    want = eng.llma_debug_logits().reshape(B, k + 1, -1)[:, 0]
+    for turn in range(20):
+        for s in range(B):
+            eng.llma_rewind(s)
+        trace, left = [], N
+        while left:
+            rows = int(rng.choice([1, 4, 5, 8, 9, 10]))
+            out = min(left, int(rng.integers(1, rows + 1)))
+            trace.append((rows, out))
+            left -= out
+        st = eng.llma_generate_forced(-1, trace, y)
+        assert st.steps == B * len(trace)
+        eng.llma_step(1, 0)
+        assert np.array_equal(eng.llma_debug_logits().reshape(B, k + 1, -1)[:, 0], want)
+    eng.llma_destroy()
