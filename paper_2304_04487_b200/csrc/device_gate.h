@@ -1,0 +1,57 @@
+// Turns of kernels whose CTAs wait for one another (library-private).
+//
+// A whole-step launch (step_simt.cu) and a projection that adds up partial tiles (gemm_tcgen05.cu, gemm_wide.cu) need all of their CTAs on
+// the GPU before any of them can finish.  The GPU gives SMs that come free to CTAs of several streams in turn, so one kernel of each kind
+// can end up with some of the SMs each and wait for the others' until its waits run out: a whole-step engine beside a tensor-core engine
+// did, within milliseconds of starting both.  So launches of the two kinds from different streams take turns: whoever launches has its
+// stream wait for what calls under way on other streams have launched of the other kind.  (Projections of several streams go on side by
+// side, as do kernels without such waits.)  Only engines of one device concern each other, and only where one takes whole steps.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <mutex>
+
+namespace llma {
+
+enum : int { kTurnNone = -1, kTurnTiles = 0, kTurnSteps = 1 };  // what is launched: nothing that waits, one kind, the other
+
+struct GateMember {  // an engine
+    int device = -1;
+    cudaStream_t stream = nullptr;
+    bool steps = false;                            // takes whole steps
+    cudaEvent_t ev[2] = {nullptr, nullptr};        // behind its last launches of each kind
+    bool in_call = false, launched[2] = {false, false};  // a call is under way, and has launched kernels of the kind
+    unsigned calls = 0;                                  // begun so far
+};
+
+// (An engine that takes whole steps waits for the calls under way: they may have launched without taking turns.)
+cudaError_t gate_join(GateMember* m, int device, cudaStream_t stream, bool steps);
+void gate_quit(GateMember* m);
+bool gate_shared(const GateMember& m);  // engines of the other kind may want turns: launch few steps at a time
+
+// A call under way.  Calls wait for what they have launched before they return, so nobody waits for a member without one.
+class GateCall {
+public:
+    explicit GateCall(GateMember& m);
+    ~GateCall();
+private:
+    GateMember& m_;
+};
+
+// Held while kernels of a kind are launched; error() after construction and end().
+class GateTurn {
+public:
+    GateTurn(GateMember& m, int kind);
+    // a call that is no engine's (kTurnTiles): the turn lasts until its destruction, which the caller's wait for the stream precedes
+    GateTurn(int device, cudaStream_t stream);
+    cudaError_t error() const { return err_; }
+    cudaError_t end();  // everything has been launched
+private:
+    void wait_for_others(const GateMember* self, cudaStream_t stream, int kind);
+    std::unique_lock<std::mutex> lock_;
+    GateMember* m_ = nullptr;
+    int device_, kind_;
+    cudaError_t err_ = cudaSuccess;
+};
+
+}  // namespace llma

@@ -51,6 +51,7 @@ static void free_prompt_buffers(llma_engine* e) {
 
 static void free_engine(llma_engine* e) {
     if (!e) return;
+    gate_quit(&e->gate);
     for (auto* graphs : {&e->step_graphs, &e->lone_graphs})
         for (auto& kv : *graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     cudaFree(e->seq_state); cudaFree(e->rows); cudaFree(e->ref);
@@ -377,6 +378,7 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     for (int i = 0; i < 2; ++i) CREATE_TRY(cudaEventCreateWithFlags(&e->ref_ev[i], cudaEventDisableTiming));
     CREATE_TRY(cudaEventCreate(&e->ev0));
     CREATE_TRY(cudaEventCreate(&e->ev1));
+    CREATE_TRY(gate_join(&e->gate, dev, e->stream, e->step_simt));
     CREATE_TRY(cudaDeviceSynchronize());
 #undef CREATE_TRY
     llma::gemm_count_engine(dev, 1);

@@ -6,6 +6,7 @@
 
 #include "../../include/llma.h"
 #include "attention_mma.cuh"
+#include "device_gate.h"
 #include "gemm_tcgen05.cuh"
 #include "kernels.h"
 #include "step_simt.cuh"
@@ -88,6 +89,8 @@ struct llma_engine {
     uint32_t* grid_barrier = nullptr;
     uint32_t ll_epoch = 1;                    // first number of the next launch
 
+    llma::GateMember gate;                    // turns with the other engines of the device
+
     // replay of a given step sequence (llma_generate_forced)
     int32_t *trace = nullptr, *target = nullptr;
     int32_t trace_cap = 0;
@@ -133,6 +136,11 @@ constexpr int kCaptureAt = 16;
 // Steps of one launch of a whole-step kernel, which ends by itself once there is nothing left to do: enough that launching costs
 // nothing (5 us against 32 steps of 20 us and more), few enough that other streams get the GPU every millisecond or so.
 constexpr int kStepsPerLaunch = 32;
+// Steps that an engine launches at a time where engines of the other kind wait for their turns (device_gate.h).  Decodes per second of two
+// engines side by side, as launches that overlapped -> turns of 8 steps (turns of 32 whole steps): two fp32 layers of width 256 beside two
+// 7B-shaped layers 143 and 150 -> 233 and 129 (397 and 89), beside two bf16 layers of width 1024 320 and 379 -> 411 and 229 (567
+// and 127).  The first engine alone: 721 a second, 684 with a look at its state every 8 steps.
+constexpr int kStepsPerTurn = 8;
 constexpr size_t kLogitStage = 1u << 17;  // floats
 int sync_state(llma_engine* e);  // h_state up to date
 void gemm_count_engine(int dev, int by);  // the last engine of a device takes the scratch that llma_gemm_rows32_bf16 keeps with it

@@ -466,6 +466,11 @@ static int capture(llma_engine* e, cudaGraphExec_t* out, Enqueue enqueue) {
     return LLMA_OK;
 }
 
+// How this engine's decoding steps wait inside a launch (device_gate.h)
+static int turn_kind(const llma_engine* e, bool whole) {
+    return whole ? kTurnSteps : (e->gemm_impl == LLMA_GEMM_TCGEN05 ? kTurnTiles : kTurnNone);
+}
+
 static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
     if (e->step_simt) return enqueue_whole_steps(e, n, k, 1, true, false);
     auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
@@ -511,10 +516,16 @@ extern "C" int llma_step(llma_engine* e, int32_t n, int32_t k, int32_t* out_toke
         const int32_t target = std::min(e->y_cap, S.y_len + (d.max_seq - S.kv_len));
         if (S.target_len != target || S.done) { S.target_len = target; S.done = 0; e->state_dirty = true; }
     }
+    GateCall call(e->gate);
     rc = push_state(e);
     if (rc) return rc;
-    rc = enqueue_lone_step(e, n, k);
-    if (rc) return rc;
+    {
+        GateTurn turn(e->gate, turn_kind(e, e->step_simt));
+        CU_TRY(turn.error());
+        rc = enqueue_lone_step(e, n, k);
+        if (rc) return rc;
+        CU_TRY(turn.end());
+    }
     // the tokens a step can have emitted come back with the state
     rc = copy_tokens(e, y_lo, y_hi);
     if (rc) return rc;
@@ -593,6 +604,9 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         e->state_dirty = true;
     }
     const bool whole = e->step_simt;
+    GateCall call(e->gate);
+    const int kind = turn_kind(e, whole);
+    const bool shared = kind != kTurnNone && gate_shared(e->gate);  // few steps at a time: other engines' turns come between
     cudaGraphExec_t graph = nullptr;
     if (!whole) {
         rc = get_step_graph(e, n, k, &graph);
@@ -622,17 +636,22 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
             if (S.active && !S.done) left = std::max(left, S.target_len - S.y_len);
         }
         if (left <= 0) break;
-        const int batch = (left + k) / (k + 1);
+        int batch = (left + k) / (k + 1);
+        GateTurn turn(e->gate, kind);
+        CU_TRY(turn.error());
         if (whole) {
             const int64_t before = e->launch_counter;
-            rc = enqueue_whole_steps(e, n, k, std::min(left, std::max(kStepsPerLaunch, 2 * batch)), !stepped, true);
+            const int most = shared ? kStepsPerTurn : std::max(kStepsPerLaunch, 2 * batch);
+            rc = enqueue_whole_steps(e, n, k, std::min(left, most), !stepped, true);
             launches += e->launch_counter - before;
             e->launch_counter = before;
         } else {
+            if (shared) batch = std::min(batch, kStepsPerTurn);
             rc = launch_steps(e, graph, n, k, batch);
             launches += (int64_t)batch * e->launches_per_step;
         }
         if (rc) return rc;
+        CU_TRY(turn.end());
         stepped = true;
         // the last look at the state brings the tokens too (a few kilobytes at most: it may be any look)
         const bool with_tokens = (size_t)(y_hi - y_lo) * d.max_batch <= 16384;
@@ -722,22 +741,33 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
     rc = push_state(e);
     if (rc) return rc;
     CU_TRY(cudaStreamSynchronize(e->stream));  // the host arrays may go after this
+    const bool whole = e->step_simt;
+    GateCall call(e->gate);
     cudaGraphExec_t graph = nullptr;
-    if (!e->step_simt) {
+    if (!whole) {
         rc = get_step_graph(e, 1, 0, &graph);
         if (rc) return rc;
     }
     CU_TRY(cudaEventRecord(e->ev0, e->stream));
     const int64_t before = e->launch_counter;
-    if (e->step_simt) rc = enqueue_whole_steps(e, 1, 0, n_steps, true, true);
-    else enqueue_tail(e, 1, 0, false, true);
+    const int kind = turn_kind(e, whole);
+    const bool shared = kind != kTurnNone && gate_shared(e->gate);
+    if (!whole) enqueue_tail(e, 1, 0, false, true);
     int64_t launches = e->launch_counter - before;
-    e->launch_counter = before;
-    if (!e->step_simt) {
-        rc = launch_steps(e, graph, 1, 0, n_steps);
-        launches += (int64_t)n_steps * e->launches_per_step;
+    for (int at = 0; at < n_steps;) {
+        const int now = std::min(n_steps - at, shared ? kStepsPerTurn : n_steps);
+        if (at > 0) CU_TRY(cudaStreamSynchronize(e->stream));
+        GateTurn turn(e->gate, kind);
+        CU_TRY(turn.error());
+        e->launch_counter = before;
+        if (whole) rc = enqueue_whole_steps(e, 1, 0, now, at == 0, true);
+        else rc = launch_steps(e, graph, 1, 0, now);
+        if (rc) return rc;
+        launches += whole ? e->launch_counter - before : (int64_t)now * e->launches_per_step;
+        CU_TRY(turn.end());
+        at += now;
     }
-    if (rc) return rc;
+    e->launch_counter = before;
     CU_TRY(cudaEventRecord(e->ev1, e->stream));
     rc = pull_state(e);
     if (rc) return rc;
@@ -775,7 +805,7 @@ extern "C" int llma_profile_steps(llma_engine* e, int32_t n, int32_t k, int32_t 
     if (rc) return rc;
     if (steps < 1) return LLMA_ERR_ARG;
     std::memset(out, 0, sizeof(*out));
-    std::vector<int32_t> toks((size_t)e->dims.max_batch * e->dims.kp1), cnt((size_t)e->dims.max_batch);
+    GateCall call(e->gate);
     for (int i = 0; i < steps; ++i) {
         // same state handling as llma_step, but the launches are bracketed by events
         rc = sync_state(e);
@@ -795,11 +825,14 @@ extern "C" int llma_profile_steps(llma_engine* e, int32_t n, int32_t k, int32_t 
         if (rc) return rc;
         e->prof_on = true;
         e->prof_n = 0;
+        GateTurn turn(e->gate, turn_kind(e, false));
+        CU_TRY(turn.error());
         mark(e, -1);
         enqueue_tail(e, n, k, false, true);
         enqueue_step_body(e, n, k, false);
         e->prof_on = false;
         CU_TRY(cudaGetLastError());
+        CU_TRY(turn.end());
         rc = pull_state(e);
         if (rc) return rc;
         rc = check_device_error(e);

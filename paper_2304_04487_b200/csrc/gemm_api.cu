@@ -129,11 +129,14 @@ extern "C" int llma_gemm_rows32_bf16(const void* W, const void* a, float* out, i
     const int grid = gemm_grid_for((int64_t)((n_out + 127) / 128) * (k_in / 64), sms);
     // the kernel reaches the page-locked word through its device address
     int32_t* err_dev = nullptr;
-    cudaError_t ce = cudaHostGetDevicePointer((void**)&err_dev, b.err, 0);
+    GateTurn turn(dev, st);  // until the wait below is over
+    cudaError_t ce = turn.error();
+    if (ce == cudaSuccess) ce = cudaHostGetDevicePointer((void**)&err_dev, b.err, 0);
     if (ce == cudaSuccess) rc = gemm_rows32_launch(W, a, out, n_out, k_in, b.ws, err_dev, grid, st);
     if (ce == cudaSuccess && rc == LLMA_OK) ce = cudaStreamSynchronize(st);  // synchronous: the block is free again after this
     const bool clean = ce == cudaSuccess && (rc == LLMA_OK || rc == LLMA_ERR_ARG) && *(volatile int32_t*)b.err == kDevErrNone;
     if (ce == cudaSuccess && rc == LLMA_OK && !clean) rc = LLMA_ERR_DEVICE_TIMEOUT;
+    turn.end();
     {
         std::lock_guard<std::mutex> lock(d.mu);
         if (clean && d.idle.size() < kMaxIdle) { d.idle.push_back(b); b = Block(); }

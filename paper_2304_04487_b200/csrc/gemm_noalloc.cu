@@ -84,6 +84,8 @@ extern "C" int llma_gemm_rows32_bf16_noalloc(const void* W, const void* a, float
         }
     } leave{sc};
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    GateTurn turn(dev, st);  // until the call returns
+    CU_TRY(turn.error());
     int grid = gemm_grid_for((int64_t)n_tiles * (k_in / 64), sms);
     if (grid > kMaxGrid) grid = kMaxGrid;
     // A call leaves the hand-over slots empty (all-ones words), as it needs them.  After one that did not end well, and for the first, all of them

@@ -1,0 +1,86 @@
+"""Engines of both kinds side by side, each with a thread and a stream of its own: every call gives what it gives alone."""
+import threading
+import time
+
+import pytest
+
+from workloads import SHAPES, build_reference, make_prompt, make_weights
+
+pytestmark = pytest.mark.gpu
+
+
+def _engine(name, k, impl=0):
+    from paper_2304_04487_b200 import Engine
+    shape = SHAPES[name]
+    eng = Engine(shape, make_weights(shape, seed=0), max_seq=220, max_ref=128, max_k=k, gemm_impl=impl)
+    eng.llma_prefill(0, make_prompt(100, shape.vocab, seed=1))
+    (y,), _ = eng.llma_generate(48, 1, 0)
+    ref, offs, _ = build_reference(y, [128], 0.7, shape.vocab, seed=0)
+    eng.llma_set_reference(0, ref, offs)
+    return eng, y
+
+
+def _generate(eng, y, k):
+    eng.llma_rewind(0)
+    (toks,), _ = eng.llma_generate(48, 1, k)
+    assert toks == y
+
+
+def _step(eng, y, k):
+    eng.llma_rewind(0)
+    got = []
+    while len(got) < 48:
+        got += eng.llma_step(1, k)[0]
+    assert got[:48] == y
+
+
+def _replay(eng, y, k):
+    eng.llma_rewind(0)
+    assert eng.llma_generate_forced(0, [(1, 1)] * 24 + [(3, 2)] * 12, y).tokens == 48
+    eng.llma_rewind(0)
+    eng.llma_profile_steps(1, k, 3)
+
+
+def _product(noalloc):
+    import torch
+    from paper_2304_04487_b200 import llma_gemm_rows32_bf16, llma_gemm_rows32_bf16_noalloc
+    gemm = llma_gemm_rows32_bf16_noalloc if noalloc else llma_gemm_rows32_bf16
+    g = torch.Generator(device="cuda").manual_seed(2)
+    W = (torch.randn(4096, 4096, device="cuda", generator=g) * 0.02).to(torch.bfloat16)
+    a = torch.randn(32, 4096, device="cuda", generator=g).to(torch.bfloat16)
+    want, out, st = torch.empty(32, 4096, device="cuda"), torch.empty(32, 4096, device="cuda"), torch.cuda.Stream()
+    gemm(W, a, want)
+    torch.cuda.synchronize()
+
+    def work():
+        gemm(W, a, out, stream=st)
+        with torch.cuda.stream(st):
+            assert torch.equal(out, want)
+    return work
+
+
+@pytest.mark.parametrize("whole,tiles", [("tiny-fp32", "mid-bf16"), ("small-bf16", "mid-bf16"), ("tiny-bf16", "llama7b-1layer")])
+def test_whole_steps_beside_other_engines(whole, tiles):
+    a, ya = _engine(whole, 4)
+    b, yb = _engine(whole, 4)
+    c, yc = _engine(tiles, 8)
+    jobs = [lambda: (_generate(a, ya, 4), _replay(a, ya, 4)), lambda: (_step(b, yb, 4), _generate(b, yb, 4)),
+            lambda: (_generate(c, yc, 8), _step(c, yc, 8), _replay(c, yc, 8)), _product(False), _product(True)]
+    failed, done, until = [], [0] * len(jobs), time.monotonic() + 1.0
+
+    def loop(i):
+        try:
+            while time.monotonic() < until and not failed:
+                jobs[i]()
+                done[i] += 1
+        except Exception as e:  # noqa: BLE001 (a thread's failure is the test's)
+            failed.append((i, e))
+
+    threads = [threading.Thread(target=loop, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed and min(done) > 0, (failed, done)
+    for e in (a, b, c):
+        e.llma_destroy()
