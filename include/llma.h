@@ -228,7 +228,9 @@ int llma_generate_forced(llma_engine *e, int32_t seq, const int32_t *trace, int3
                          const int32_t *target, int32_t n_target, llma_stats *stats);
 
 /* Parity harness only: preset the device-side error word (0 none, 1 a bounded wait ran out, 2 capacity,
- * 3 token range), as a kernel that gave up would have left it; the next step reports it.  Errors: ARG, CUDA. */
+ * 3 token range), as a kernel that gave up would have left it; the next step reports it.  4: a launch of whole decoding steps has given
+ * up because its CTAs did not get onto the GPU together; engines that take whole steps repeat it, for 30 seconds before they report
+ * DEVICE_TIMEOUT.  Errors: ARG, CUDA. */
 int llma_debug_set_device_error(llma_engine *e, int32_t code);
 
 /* Measurement aid: in-kernel timestamps of the last decoding step's kernels (globaltimer, ns), copied to `out`

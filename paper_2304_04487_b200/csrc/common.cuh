@@ -64,6 +64,7 @@ enum : int32_t {
     kDevErrTimeout = 1,   // a bounded wait ran out
     kDevErrCapacity = 2,  // a step would have written past max_seq
     kDevErrToken = 3,     // a token id out of range reached the device
+    kDevErrSteps = 4,     // a launch of whole steps has given up and may be repeated
 };
 
 struct ModelDims {

@@ -1,5 +1,6 @@
 // Decoding entry points of the C ABI: prefill, reference upload, step, generate.
 #include <algorithm>
+#include <chrono>
 #include <climits>
 #include <cstring>
 #include <vector>
@@ -203,23 +204,20 @@ static void enqueue_step_body(llma_engine* e, int n, int k, bool plan_next) {
     enqueue_tail(e, n, k, true, plan_next);
 }
 
-// Up to `steps` decoding steps as launches of the whole-step kernel (fewer if no sequence has anything left to do).  plan_first: plan
-// the first one (otherwise the launch before has planned it); plan_last: plan the step after the last one.
-static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps, bool plan_first, bool plan_last) {
+// Up to `steps` decoding steps as launches of the whole-step kernel (fewer if no sequence has anything left to do), each with its plan
+static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps) {
     SimtStep s = e->simt;
     e->plain_acts = true;
     s.tail = tail_args(e, n, k);
     const uint32_t per_step = simt_epochs(e->dims);
-    for (; steps > 0; steps -= kStepsPerLaunch, plan_first = false) {
+    for (; steps > 0; steps -= kStepsPerLaunch) {
         s.max_steps = std::min(steps, kStepsPerLaunch);
-        s.plan_first = plan_first ? 1 : 0;
-        s.plan_last = plan_last || steps > kStepsPerLaunch ? 1 : 0;
         if (e->ll_epoch > 0xFFFFFFFFu - per_step * (kStepsPerLaunch + 2)) {  // the numbers begin again
             CU_TRY(cudaMemsetAsync(e->ll_words, 0, e->ll_count * sizeof(unsigned long long), e->stream));
             e->ll_epoch = 1;
         }
         s.epoch = e->ll_epoch;
-        e->ll_epoch += per_step * (uint32_t)(s.max_steps + 1);  // (the rows of the step after the last one are published too)
+        e->ll_epoch += per_step * (uint32_t)s.max_steps;
         CU_TRY(launch_step_simt(e->stream, e->bf16, s, e->simt_smem, e->num_sms));
         e->launch_counter += 1;
     }
@@ -270,12 +268,28 @@ static int check_device_error(llma_engine* e) {
     // a kernel that gave up may have left partial tiles in the hand-over slots: empty them again, so that
     // a caller who carries on after the error does not sum stale partials into later projections
     if (code == kDevErrTimeout && e->gemm_ws) CU_TRY(cudaMemsetAsync(e->gemm_ws, 0xFF, e->gemm_ws_bytes, e->stream));
-    if (code == kDevErrTimeout && e->grid_barrier) CU_TRY(cudaMemsetAsync(e->grid_barrier, 0, sizeof(uint32_t), e->stream));
+    if (e->grid_barrier) CU_TRY(cudaMemsetAsync(e->grid_barrier, 0, sizeof(uint32_t), e->stream));
     CU_TRY(cudaStreamSynchronize(e->stream));
     *e->h_err = kDevErrNone;
-    if (code == kDevErrTimeout) return LLMA_ERR_DEVICE_TIMEOUT;
+    if (code == kDevErrTimeout || code == kDevErrSteps) return LLMA_ERR_DEVICE_TIMEOUT;
     if (code == kDevErrCapacity) return LLMA_ERR_CAPACITY;
     return LLMA_ERR_TOKEN_RANGE;
+}
+
+// After pull_state: whether launches of whole steps have given up and are to be repeated.  They do when something else keeps SMs from
+// their CTAs for long; the state is then that after the last step that was whole, and the words and rows of the unfinished one
+// are written again.  For half a minute at most, after which the error is reported.
+static int whole_steps_again(llma_engine* e, std::chrono::steady_clock::time_point* since, bool* again) {
+    *again = false;
+    if (*e->h_err != kDevErrSteps) return LLMA_OK;
+    const auto now = std::chrono::steady_clock::now();
+    if (since->time_since_epoch().count() == 0) *since = now;
+    if (now - *since > std::chrono::seconds(30)) return LLMA_OK;
+    CU_TRY(cudaMemsetAsync(e->dev_err, 0, sizeof(int32_t), e->stream));
+    CU_TRY(cudaMemsetAsync(e->grid_barrier, 0, sizeof(uint32_t), e->stream));
+    *e->h_err = kDevErrNone;
+    *again = true;
+    return LLMA_OK;
 }
 
 // Positions p0 .. p0 + n - 1 of a prompt (tokens in e->p_tok) through the decoder, into the K/V cache.  Nothing but the cache
@@ -472,7 +486,7 @@ static int turn_kind(const llma_engine* e, bool whole) {
 }
 
 static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
-    if (e->step_simt) return enqueue_whole_steps(e, n, k, 1, true, false);
+    if (e->step_simt) return enqueue_whole_steps(e, n, k, 1);
     auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
     llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k);
     if (!e->can_capture || g.uses + 1 < kCaptureAt) {
@@ -519,18 +533,25 @@ extern "C" int llma_step(llma_engine* e, int32_t n, int32_t k, int32_t* out_toke
     GateCall call(e->gate);
     rc = push_state(e);
     if (rc) return rc;
-    {
+    std::chrono::steady_clock::time_point gave_up{};
+    for (bool again = true; again;) {
         GateTurn turn(e->gate, turn_kind(e, e->step_simt));
         CU_TRY(turn.error());
         rc = enqueue_lone_step(e, n, k);
         if (rc) return rc;
         CU_TRY(turn.end());
+        // the tokens a step can have emitted come back with the state
+        rc = copy_tokens(e, y_lo, y_hi);
+        if (rc) return rc;
+        rc = pull_state(e);
+        if (rc) return rc;
+        again = false;
+        if (e->step_simt) {
+            rc = whole_steps_again(e, &gave_up, &again);
+            if (rc) return rc;
+            for (int s = 0; s < d.max_batch; ++s) again = again && e->h_state[s].y_len == y0[s];  // (the step itself may have been whole)
+        }
     }
-    // the tokens a step can have emitted come back with the state
-    rc = copy_tokens(e, y_lo, y_hi);
-    if (rc) return rc;
-    rc = pull_state(e);
-    if (rc) return rc;
     rc = check_device_error(e);
     if (rc) return rc;
     for (int s = 0; s < d.max_batch; ++s) {
@@ -621,6 +642,7 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
     // (A launch of the whole-step kernel ends by itself when there is nothing left to do: twice that many may be asked for.)
     int64_t launches = 0;
     bool have_tokens = false, stepped = false;
+    std::chrono::steady_clock::time_point gave_up{};
     CU_TRY(cudaEventRecord(e->ev0, e->stream));
     // the first step's plan; every graph launch then ends with the plan of the step after it
     if (!whole || max_new == 0) {
@@ -642,7 +664,7 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         if (whole) {
             const int64_t before = e->launch_counter;
             const int most = shared ? kStepsPerTurn : std::max(kStepsPerLaunch, 2 * batch);
-            rc = enqueue_whole_steps(e, n, k, std::min(left, most), !stepped, true);
+            rc = enqueue_whole_steps(e, n, k, std::min(left, most));
             launches += e->launch_counter - before;
             e->launch_counter = before;
         } else {
@@ -660,6 +682,11 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         rc = pull_state(e);
         if (rc) return rc;
         have_tokens = with_tokens;
+        if (whole) {
+            bool again;
+            rc = whole_steps_again(e, &gave_up, &again);
+            if (rc) return rc;
+        }
         if (*e->h_err != kDevErrNone) break;
     }
     if (!stepped) {  // no step was taken
@@ -754,23 +781,29 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
     const bool shared = kind != kTurnNone && gate_shared(e->gate);
     if (!whole) enqueue_tail(e, 1, 0, false, true);
     int64_t launches = e->launch_counter - before;
-    for (int at = 0; at < n_steps;) {
-        const int now = std::min(n_steps - at, shared ? kStepsPerTurn : n_steps);
-        if (at > 0) CU_TRY(cudaStreamSynchronize(e->stream));
-        GateTurn turn(e->gate, kind);
-        CU_TRY(turn.error());
+    std::chrono::steady_clock::time_point gave_up{};
+    for (bool again = true; again;) {
+        for (int at = 0; at < n_steps;) {
+            const int now = std::min(n_steps - at, shared ? kStepsPerTurn : n_steps);
+            if (at > 0) CU_TRY(cudaStreamSynchronize(e->stream));
+            GateTurn turn(e->gate, kind);
+            CU_TRY(turn.error());
+            e->launch_counter = before;
+            if (whole) rc = enqueue_whole_steps(e, 1, 0, now);
+            else rc = launch_steps(e, graph, 1, 0, now);
+            if (rc) return rc;
+            launches += whole ? e->launch_counter - before : (int64_t)now * e->launches_per_step;
+            CU_TRY(turn.end());
+            at += now;
+        }
         e->launch_counter = before;
-        if (whole) rc = enqueue_whole_steps(e, 1, 0, now, at == 0, true);
-        else rc = launch_steps(e, graph, 1, 0, now);
+        CU_TRY(cudaEventRecord(e->ev1, e->stream));
+        rc = pull_state(e);
         if (rc) return rc;
-        launches += whole ? e->launch_counter - before : (int64_t)now * e->launches_per_step;
-        CU_TRY(turn.end());
-        at += now;
+        again = false;
+        if (whole) rc = whole_steps_again(e, &gave_up, &again);  // (launches beyond the trace's end find nothing to do)
+        if (rc) return rc;
     }
-    e->launch_counter = before;
-    CU_TRY(cudaEventRecord(e->ev1, e->stream));
-    rc = pull_state(e);
-    if (rc) return rc;
     rc = check_device_error(e);
     if (rc) return rc;
     llma_stats st;
@@ -793,7 +826,7 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
 
 extern "C" int llma_debug_set_device_error(llma_engine* e, int32_t code) {
     if (!e) return LLMA_ERR_NULL;
-    if (code < kDevErrNone || code > kDevErrToken) return LLMA_ERR_ARG;
+    if (code < kDevErrNone || code > kDevErrSteps) return LLMA_ERR_ARG;
     CU_TRY(cudaMemcpyAsync(e->dev_err, &code, sizeof(int32_t), cudaMemcpyHostToDevice, e->stream));
     CU_TRY(cudaStreamSynchronize(e->stream));
     return LLMA_OK;

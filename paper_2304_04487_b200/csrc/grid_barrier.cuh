@@ -22,13 +22,13 @@ struct GridBarrier {
         const uint32_t add = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u;
         asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(word), "r"(add) : "memory");
     }
-    __device__ __forceinline__ bool wait() {
+    __device__ __forceinline__ bool wait(uint64_t most_ns) {
         const uint32_t old = sense;
         sense ^= 0x80000000u;
         const uint64_t t0 = ptx::globaltimer_ns();
         do {
             if ((ptx::ld_acquire(word) ^ old) & 0x80000000u) return true;
-        } while (ptx::globaltimer_ns() - t0 < 2000000000ull);
+        } while (ptx::globaltimer_ns() - t0 < most_ns);
         return false;
     }
 };

@@ -67,17 +67,32 @@ __device__ __forceinline__ LL2 ll_load2(const LLWord* p) {
 }
 __device__ __forceinline__ bool ll_ready(const LL2& w, uint32_t epoch) { return (uint32_t)(w.a >> 32) == epoch && (uint32_t)(w.b >> 32) == epoch; }
 __device__ __forceinline__ float2 ll_values(const LL2& w) { return make_float2(__uint_as_float((uint32_t)w.a), __uint_as_float((uint32_t)w.b)); }
+// A wait runs out when the launch's CTAs are not on the GPU together, because something else holds SMs for long.  Such a launch is as
+// good as not made: CTA 0 writes no state back, what else has been written belongs to positions that the state does not reach, and
+// the host launches its steps again.  The mark is on its way before anything that is made of what has not arrived, so CTA 0 finds it once
+// it has a result that depends on that.  (Keeping such results from being published instead, by barriers that tell all threads of a
+// CTA, cost 0.4 to 1.5 us a step.)
+struct GiveUp {
+    volatile int* failed;  // of the CTA
+    int32_t* mark;         // the device error word
+    int patience;          // polls
+    __device__ __forceinline__ void now() const {
+        atomicExch(mark, kDevErrSteps);
+        __threadfence();
+        *failed = 1;
+    }
+};
 // Polls until every pair of words carries the number: at(u) is where pair u lies, nullptr if there is none.  The pairs that are missing are
-// fetched together, so that the wait ends a trip to L2 after the last of them has landed.  Bounded (about two seconds): raises the
-// CTA's flag when the wait runs out, and no wait of the CTA lasts once it is up.
+// fetched together, so that the wait ends a trip to L2 after the last of them has landed.  Bounded: the CTA gives up when the wait runs
+// out, and no wait of the CTA lasts once it has.
 template <int U, typename At>
-__device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, volatile int* failed, At at) {
+__device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, const GiveUp& up, At at) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         w[u].a = w[u].b = (LLWord)epoch << 32;
         if (const LLWord* p = at(u)) w[u] = ll_load2(p);
     }
-    int left = 1 << 22;
+    int left = up.patience;
 #pragma unroll 1
     for (;;) {
         bool all = true;
@@ -89,17 +104,17 @@ __device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, volatile i
             }
         }
         if (all) break;
-        if (--left == 0) *failed = 1;
-        if (*failed) break;
+        if (--left == 0) up.now();
+        if (*up.failed) break;
     }
 }
-__device__ __forceinline__ void ll_wait2(LL2& w, const LLWord* p, uint32_t epoch, volatile int* failed) {  // w has been fetched once
-    int left = 1 << 22;
+__device__ __forceinline__ void ll_wait2(LL2& w, const LLWord* p, uint32_t epoch, const GiveUp& up) {  // w has been fetched once
+    int left = up.patience;
 #pragma unroll 1
     while (!ll_ready(w, epoch)) {
         w = ll_load2(p);
-        if (--left == 0) *failed = 1;
-        if (*failed) break;
+        if (--left == 0) up.now();
+        if (*up.failed) break;
     }
 }
 
@@ -155,7 +170,7 @@ template <int N> __device__ __forceinline__ void load_few(bool cached, const __n
 // sm: q, the sequence's own K and V rows of the step, then the warps' partial results.
 template <typename T, int HD>
 __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int layer, int head, int r, uint32_t epoch, float* sm,
-                                       volatile int* failed) {
+                                       const GiveUp& up) {
     constexpr int NJ = HD / 32;   // float4 of k per lane of an eight-lane group
     constexpr int NF = HD / 32;   // output values per lane
     const ModelDims& dims = a.dims;
@@ -176,7 +191,7 @@ __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int
             const int s = i / P, c = 2 * (i % P);  // 0 q; then k and v of a row in turn
             const int row = r - (s > 0 ? (s - 1) >> 1 : 0), part = s == 0 ? 0 : 2 - (s & 1);
             LL2 w[1];
-            ll_fetch(w, epoch, failed, [&](int) { return words + (3 * row + part) * HT + c; });
+            ll_fetch(w, epoch, up, [&](int) { return words + (3 * row + part) * HT + c; });
             const float2 v = ll_values(w[0]);
             if (s == 0) {
                 *reinterpret_cast<float2*>(s_q + c) = v;
@@ -271,8 +286,12 @@ __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int
     workers_sync();
 }
 
+// The launch before has given up: this one would meet the barrier half passed, and its steps are launched again anyway.  (A CTA that only
+// gets an SM when others of its own launch have given up may see it too.)
+__device__ __forceinline__ bool given_up(const SimtStep& a) { return threadIdx.x == 0 && __ldcg(a.dev_err) == kDevErrSteps; }
+
 // Acceptance and plan, step after step (CTA 0)
-__device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatile int* failed) {
+__device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const GiveUp& up) {
     const ModelDims& d = a.dims;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = d.max_batch;
     const int n_parts = min((int)gridDim.x - 1, a.geo[kOpHead].n_units);
@@ -284,8 +303,6 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatil
     v.ref = v.tok + d.row_cap;
     v.y = v.ref + B * 3 * d.max_ref;
     for (int i = tid; i < B * kStateWords; i += kThreads) reinterpret_cast<int*>(v.st)[i] = __ldcg(reinterpret_cast<const int*>(a.tail.st) + i);
-    for (int s = tid; s < B; s += kThreads) v.first[s] = __ldcg(&a.rows->seq_first[s]);
-    if (tid == 0) v.first[B] = __ldcg(&a.rows->rows_used);
     __syncthreads();
 #pragma unroll 1
     for (int s = 0; s < B; ++s) {
@@ -297,6 +314,7 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatil
 #pragma unroll 1
         for (int i = tid; i < v.st[s].y_len; i += kThreads) v.y[s * a.tail.y_cap + i] = __ldcg(a.tail.y + (int64_t)s * a.tail.y_cap + i);
     }
+    if (__syncthreads_or(given_up(a))) return;
     GridBarrier bar(a.barrier);
     uint32_t epoch = a.epoch;
     auto publish = [&](int r, int tok, int pos, int seq, int first) {
@@ -306,17 +324,17 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatil
     };
     auto publish_count = [&](int used) { ll_store2(ll_rows_of(a, epoch), __int_as_float(used), 0.f, epoch); };
     __syncthreads();
-    // step -1: the plan of the first step, or what the launch before has planned
+    // step -1: the plan of the first step
 #pragma unroll 1
     for (int step = -1; step < a.max_steps; ++step) {
         TailArgs t = a.tail;
-        t.do_accept = 0; t.do_plan = a.plan_first;
+        t.do_accept = 0; t.do_plan = 1;
         if (step >= 0) {
             const bool last = step + 1 == a.max_steps;
             const int rows_used = v.first[B];
             if (rows_used == 0) break;
             if (tid == 0) {  // rows are published into the other half of ll_rows: every CTA has read what was there
-                if (step > 0 && !bar.wait()) *failed = 1;
+                if (step > 0 && !bar.wait(600ull * a.patience)) up.now();
                 if (!last) bar.arrive();
             }
 #pragma unroll 1
@@ -326,7 +344,7 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatil
 #pragma unroll 1
                 for (int p = lane; p < n_parts; p += 160) {
                     LL2 w[5];
-                    ll_fetch(w, epoch + 4 * d.n_layers, failed,
+                    ll_fetch(w, epoch + 4 * d.n_layers, up,
                              [&](int u) { return p + 32 * u < n_parts ? a.ll_part + 2 * ((int64_t)(p + 32 * u) * d.row_cap + r) : nullptr; });
 #pragma unroll
                     for (int u = 0; u < 5; ++u) {
@@ -343,21 +361,14 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, volatil
                 }
                 if (lane == 0) { v.tok[r] = i; a.tail.out_tok[r] = i; }
             }
-            if (__syncthreads_or(*failed)) break;
+            if (__syncthreads_or(*up.failed)) break;
             epoch += simt_epochs(d);
-            t.do_accept = 1; t.do_plan = !last || a.plan_last != 0;
-        } else if (!a.plan_first) {
-#pragma unroll 1
-            for (int r = tid; r < d.row_cap; r += kThreads) {
-                const int seq = __ldcg(&a.rows->seq[r]);
-                publish(r, __ldcg(&a.rows->tok[r]), __ldcg(&a.rows->pos[r]), seq, v.first[seq]);
-            }
-            if (tid == 0) publish_count(v.first[B]);
+            t.do_accept = 1; t.do_plan = !last;
         }
         step_tail_on<kThreads, true>(t, v, publish, publish_count);
         __syncthreads();
     }
-    if (tid == 0 && *failed) atomicExch(a.dev_err, kDevErrTimeout);
+    if (__syncthreads_or(tid == 0 && ld_acquire(reinterpret_cast<const uint32_t*>(a.dev_err)) == kDevErrSteps)) return;
     for (int i = tid; i < B * kStateWords; i += kThreads) reinterpret_cast<int*>(a.tail.st)[i] = reinterpret_cast<const int*>(v.st)[i];
 }
 
@@ -378,9 +389,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
     }
     fence_mbar_init();
     __syncthreads();
-    volatile int* const failed = &s_fail;
+    const GiveUp up = {&s_fail, a.dev_err, a.patience};
     if (blockIdx.x == 0) {
-        tail_cta(a, reinterpret_cast<uint8_t*>(sA), &s_fail);
+        tail_cta(a, reinterpret_cast<uint8_t*>(sA), up);
         return;
     }
     const ModelDims& d = a.dims;
@@ -398,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         const unsigned long long* src = reinterpret_cast<const unsigned long long*>(a.ops);
         for (int i = tid; i < n_ops * (int)(sizeof(SimtOp) / 8); i += kThreads) reinterpret_cast<unsigned long long*>(s_ops)[i] = __ldg(src + i);
     }
-    __syncthreads();
+    if (__syncthreads_or(given_up(a))) return;
     GridBarrier bar(a.barrier);
     float* s_gain = sA + a.gain_offset / 4;  // the norm's gains
 
@@ -603,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
 #pragma unroll 1
                     for (int i0 = 2 * tid; i0 < total; i0 += U * kSweep) {
                         LL2 w[U];
-                        ll_fetch(w, want, failed, [&](int u) { return i0 + u * kSweep < total ? src + i0 + u * kSweep : nullptr; });
+                        ll_fetch(w, want, up, [&](int u) { return i0 + u * kSweep < total ? src + i0 + u * kSweep : nullptr; });
 #pragma unroll
                         for (int u = 0; u < U; ++u)
                             if (i0 + u * kSweep < total) put(ll_values(w[u]));
@@ -623,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                     if (n_pieces > kRing << lg) lane_rows(unit_rows(op, m, unit), q0, q1);
 #pragma unroll 1
                     for (int c = warp & ((1 << lg) - 1); c < n_pieces; c += 1 << lg) {
-                        if (!mbar_wait(full + 8 * c_slot, c_phase)) *failed = 1;
+                        if (!mbar_wait(full + 8 * c_slot, c_phase)) up.now();
                         uint4 w0, w1;
                         {
                             const uint32_t src = ring + c_slot * 1024;
@@ -744,7 +755,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                         a.h[e_at] = v;
                     } else if (m != kOpHead) {
                         if (!(m == kOpO && op == kOpO)) {
-                            ll_wait2(ex, a.ll_x + e_at, epoch - 2, failed);  // the residual projection before this one
+                            ll_wait2(ex, a.ll_x + e_at, epoch - 2, up);  // the residual projection before this one
                             e0 = ll_values(ex).x; e1 = ll_values(ex).y;
                         }
                         ll_store2(a.ll_x + e_at, e0 + v0, e1 + v1, epoch);
@@ -797,11 +808,11 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
 #pragma unroll 1
             for (int r = tid; r < a.tail.n_rows; r += kST) {
                 LL2 v[3];
-                ll_fetch(v, epoch0, failed, [&](int u) { return u == 2 ? w : w + 2 + 4 * r + 2 * u; });
+                ll_fetch(v, epoch0, up, [&](int u) { return u == 2 ? w : w + 2 + 4 * r + 2 * u; });
                 const LL2 &x = v[0], &y = v[1], &z = v[2];
                 int tok = (int)(uint32_t)x.a;
                 if (tok < 0 || tok >= d.vocab) {
-                    if (cta == 0) atomicExch(a.dev_err, kDevErrToken);
+                    if (cta == 0) atomicCAS(a.dev_err, kDevErrNone, kDevErrToken);  // (not over the mark of a CTA that has given up)
                     tok = 0;
                 }
                 R.tok[r] = tok; R.pos[r] = (int)(uint32_t)x.b; R.seq[r] = (int)(uint32_t)y.a; R.first[r] = (int)(uint32_t)y.b;
@@ -811,7 +822,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         workers_sync();
         rows_used = R.used;
 
-        if (rows_used == 0 || *failed) break;  // nothing left to do (or a wait ran out, seconds ago)
+        if (rows_used == 0 || *up.failed) break;  // nothing left to do, or a wait ran out
         if (tid == 0 && a.passes > 1) {
             int n = 1;
             for (int r = pass; r < rows_used; r += pass) ++n;
@@ -840,12 +851,12 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                 else project(std::integral_constant<int, kSR>{}, m, op, epoch);
             }
             if (m == kOpQKV) {
-                if (op == 0 && step > 0 && tid == 0 && !bar.wait()) *failed = 1;  // the cache rows of the step before
+                if (op == 0 && step > 0 && tid == 0 && !bar.wait(600ull * a.patience)) up.now();  // the cache rows of the step before
                 workers_sync();
 #pragma unroll 1
                 for (int it = cta; it < rows_used * d.n_heads; it += G) {
                     const int r = it / d.n_heads;
-                    attend<T, HD>(a, R, op >> 2, it - r * d.n_heads, r, epoch, sA, failed);
+                    attend<T, HD>(a, R, op >> 2, it - r * d.n_heads, r, epoch, sA, up);
                 }
             }
         }
@@ -854,7 +865,6 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         if (tid == 0) bar.arrive();
     }
     *(volatile int*)&s_stop = 1;
-    if (tid == 0 && *failed) atomicExch(a.dev_err, kDevErrTimeout);
 }
 
 // ---- host side -----------------------------------------------------------------------------------------------------
@@ -879,6 +889,10 @@ bool step_simt_shape(const ModelDims& d, bool bf16, int y_cap, int num_sms, Simt
     s->gain_offset = (int)(at + kRingBytes);
     s->ops_offset = (int)(at + kRingBytes + gains);
     *smem = at + kRingBytes + gains + ops;
+    // Polls take 0.6 us and more: 20 ms, and 2.5 ms per projection and pass, some thirty times what the slowest take.  A CTA may have
+    // nothing to do for a whole step, so that is what the bound is made for.
+    const long long polls = 32768 + 4096ll * (4 * d.n_layers + 1) * passes;
+    s->patience = (int)(polls < 1 << 22 ? polls : 1 << 22);
     const size_t B = d.max_batch, tail = B * (8 + sizeof(SeqState) + 4) + 4 + ((size_t)d.row_cap + B * (3 * (size_t)d.max_ref + y_cap)) * 4;
     if (*smem < tail) *smem = (tail + 15) / 16 * 16;
     if (*smem > kStepSmem) return false;

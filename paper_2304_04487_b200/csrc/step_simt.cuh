@@ -37,8 +37,7 @@ struct SimtStep {
     int32_t passes;      // most passes of a step
     int32_t ring_offset, gain_offset, ops_offset;  // bytes of dynamic shared memory before the weight ring, a norm's gains, the ops
     int32_t max_steps;   // steps of this launch; it ends early once no sequence has anything left to do
-    int32_t plan_first;  // plan the first step (otherwise the launch before has)
-    int32_t plan_last;   // plan the step after the last one
+    int32_t patience;    // polls before a wait gives up
 };
 // numbers that a step takes: at least one per projection, and an odd number (ll_rows has a half for odd and one for even steps)
 __host__ __device__ inline uint32_t simt_epochs(const ModelDims& d) { return 4u * d.n_layers + 3u; }

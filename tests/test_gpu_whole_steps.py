@@ -93,3 +93,43 @@ def test_passes_change_from_step_to_step():
         eng.llma_step(1, 0)
         assert np.array_equal(eng.llma_debug_logits().reshape(B, k + 1, -1)[:, 0], want)
     eng.llma_destroy()
+
+
+@pytest.mark.parametrize("name", ["tiny-bf16", "tiny-fp32"])
+def test_launches_that_give_up_are_repeated(name):
+    """A launch of whole steps whose CTAs did not get onto the GPU together leaves its mark in the error word: launches behind it do
+    nothing, the call launches them again and gives what it gives undisturbed.  (The mark is preset; no wait is made to run out.)"""
+    from paper_2304_04487_b200 import Engine
+    from workloads import SHAPES
+    shape = SHAPES[name]
+    N, k = 70, 4                                                   # more than two launches
+    eng = Engine(shape, make_weights(shape, seed=0), max_seq=30 + N + k, max_ref=N, max_k=k)
+    eng.llma_prefill(0, make_prompt(20, shape.vocab, seed=1))
+    (y,), st = eng.llma_generate(N, 1, 0)
+    assert st.launches == 3
+    eng.llma_set_reference(0, y)
+
+    def generate(k):
+        (toks,), st = eng.llma_generate(N, 1, k)
+        assert toks == y and st.tokens == N and st.steps == N - st.copied_accepted
+        return st.launches
+
+    def steps():
+        got = []
+        while len(got) < N:
+            eng.llma_debug_set_device_error(4)
+            got += eng.llma_step(1, k)[0]
+        assert got[:N] == y
+
+    def replay(trace):
+        st = eng.llma_generate_forced(0, trace, y)
+        assert (st.steps, st.tokens) == (len(trace), N)
+
+    for call in (lambda: generate(0), lambda: generate(k), steps, lambda: replay([(1, 1)] * 10 + [(5, 3)] * 20)):
+        eng.llma_rewind(0)
+        eng.llma_debug_set_device_error(4)
+        call()
+    eng.llma_rewind(0)
+    eng.llma_debug_set_device_error(4)
+    assert generate(0) > 3                                         # those that did nothing, and those that did
+    eng.llma_destroy()
