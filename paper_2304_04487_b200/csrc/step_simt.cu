@@ -464,7 +464,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
         UnitRows u = {nullptr, nullptr, 0, 0};
         bool find = true, any = true;  // the unit's rows have to be found; the warp has something to multiply at all
         volatile int *stop = &s_stop, *steps = &s_steps, *passes = s_passes;
-        while (!*stop) {
+        // (what the lanes read one by one may change between them: such a decision is the warp's, or they would part for good)
+        while (!__any_sync(0xffffffffu, *stop)) {
             bool ready = any;
             if (any && unit >= units) {  // done with a pass over a projection, or not begun
                 // (how many passes a step has is known once it has begun, and is read of the step that is being fed: the next one may
@@ -503,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                 const char *q0, *q1;
                 lane_rows(v, q0, q1);
                 const int place0 = ((warp - kSW) * kEach + i) * kRing;
-                while (pc < end && mbar_test(empty0 + 8 * (place0 + sl), (ph >> sl) & 1u)) {
+                while (pc < end && __all_sync(0xffffffffu, mbar_test(empty0 + 8 * (place0 + sl), (ph >> sl) & 1u))) {
                     const uint32_t dst = ring0 + (place0 + sl) * 1024;
                     cp_async_16(dst, q0 + pc * 128);
                     cp_async_16(dst + 512, q1 + pc * 128);
