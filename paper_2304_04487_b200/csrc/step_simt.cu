@@ -68,25 +68,19 @@ __device__ __forceinline__ LL2 ll_load2(const LLWord* p) {
 __device__ __forceinline__ bool ll_ready(const LL2& w, uint32_t epoch) { return (uint32_t)(w.a >> 32) == epoch && (uint32_t)(w.b >> 32) == epoch; }
 __device__ __forceinline__ float2 ll_values(const LL2& w) { return make_float2(__uint_as_float((uint32_t)w.a), __uint_as_float((uint32_t)w.b)); }
 // A wait runs out when the launch's CTAs are not on the GPU together, because something else holds SMs for long.  Such a launch is as
-// good as not made: CTA 0 writes no state back, what else has been written belongs to positions that the state does not reach, and
-// the host launches its steps again.  The mark is on its way before anything that is made of what has not arrived, so CTA 0 finds it once
-// it has a result that depends on that.  (Keeping such results from being published instead, by barriers that tell all threads of a
-// CTA, cost 0.4 to 1.5 us a step.)
-struct GiveUp {
+// good as not made: a CTA that has given up (its flag is up) passes no further barrier, CTA 0 writes no state back unless every CTA has
+// passed the barrier that ends the last step, what else has been written belongs to positions that the state does not reach, and
+// the host launches the steps again.  (Keeping what has not arrived from being published instead, by barriers that tell all threads of a
+// CTA, cost 0.4 to 1.5 us a step; a mark in global memory ahead of it 0.3 to 1.4.)
+struct Waits {
     volatile int* failed;  // of the CTA
-    int32_t* mark;         // the device error word
     int patience;          // polls
-    __device__ __forceinline__ void now() const {
-        atomicExch(mark, kDevErrSteps);
-        __threadfence();
-        *failed = 1;
-    }
 };
 // Polls until every pair of words carries the number: at(u) is where pair u lies, nullptr if there is none.  The pairs that are missing are
 // fetched together, so that the wait ends a trip to L2 after the last of them has landed.  Bounded: the CTA gives up when the wait runs
 // out, and no wait of the CTA lasts once it has.
 template <int U, typename At>
-__device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, const GiveUp& up, At at) {
+__device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, const Waits& up, At at) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         w[u].a = w[u].b = (LLWord)epoch << 32;
@@ -104,16 +98,16 @@ __device__ __forceinline__ void ll_fetch(LL2 (&w)[U], uint32_t epoch, const Give
             }
         }
         if (all) break;
-        if (--left == 0) up.now();
+        if (--left == 0) *up.failed = 1;
         if (*up.failed) break;
     }
 }
-__device__ __forceinline__ void ll_wait2(LL2& w, const LLWord* p, uint32_t epoch, const GiveUp& up) {  // w has been fetched once
+__device__ __forceinline__ void ll_wait2(LL2& w, const LLWord* p, uint32_t epoch, const Waits& up) {  // w has been fetched once
     int left = up.patience;
 #pragma unroll 1
     while (!ll_ready(w, epoch)) {
         w = ll_load2(p);
-        if (--left == 0) up.now();
+        if (--left == 0) *up.failed = 1;
         if (*up.failed) break;
     }
 }
@@ -170,7 +164,7 @@ template <int N> __device__ __forceinline__ void load_few(bool cached, const __n
 // sm: q, the sequence's own K and V rows of the step, then the warps' partial results.
 template <typename T, int HD>
 __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int layer, int head, int r, uint32_t epoch, float* sm,
-                                       const GiveUp& up) {
+                                       const Waits& up) {
     constexpr int NJ = HD / 32;   // float4 of k per lane of an eight-lane group
     constexpr int NF = HD / 32;   // output values per lane
     const ModelDims& dims = a.dims;
@@ -291,7 +285,7 @@ __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int
 __device__ __forceinline__ bool given_up(const SimtStep& a) { return threadIdx.x == 0 && __ldcg(a.dev_err) == kDevErrSteps; }
 
 // Acceptance and plan, step after step (CTA 0)
-__device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const GiveUp& up) {
+__device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const Waits& up) {
     const ModelDims& d = a.dims;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = d.max_batch;
     const int n_parts = min((int)gridDim.x - 1, a.geo[kOpHead].n_units);
@@ -324,6 +318,7 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const G
     };
     auto publish_count = [&](int used) { ll_store2(ll_rows_of(a, epoch), __int_as_float(used), 0.f, epoch); };
     __syncthreads();
+    bool begun = false;  // thread 0: a barrier is under way
     // step -1: the plan of the first step
 #pragma unroll 1
     for (int step = -1; step < a.max_steps; ++step) {
@@ -334,8 +329,9 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const G
             const int rows_used = v.first[B];
             if (rows_used == 0) break;
             if (tid == 0) {  // rows are published into the other half of ll_rows: every CTA has read what was there
-                if (step > 0 && !bar.wait(600ull * a.patience)) up.now();
-                if (!last) bar.arrive();
+                if (step > 0 && !bar.wait(600ull * a.patience)) *up.failed = 1;
+                bar.arrive();
+                begun = true;
             }
 #pragma unroll 1
             for (int r = warp; r < rows_used; r += kThreads / 32) {  // final token: lowest index on ties
@@ -368,7 +364,11 @@ __device__ __forceinline__ void tail_cta(const SimtStep& a, uint8_t* sm, const G
         step_tail_on<kThreads, true>(t, v, publish, publish_count);
         __syncthreads();
     }
-    if (__syncthreads_or(tid == 0 && ld_acquire(reinterpret_cast<const uint32_t*>(a.dev_err)) == kDevErrSteps)) return;
+    if (begun && !bar.wait(600ull * a.patience)) *up.failed = 1;
+    if (__syncthreads_or(*up.failed)) {
+        if (tid == 0) atomicExch(a.dev_err, kDevErrSteps);
+        return;
+    }
     for (int i = tid; i < B * kStateWords; i += kThreads) reinterpret_cast<int*>(a.tail.st)[i] = reinterpret_cast<const int*>(v.st)[i];
 }
 
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
     }
     fence_mbar_init();
     __syncthreads();
-    const GiveUp up = {&s_fail, a.dev_err, a.patience};
+    const Waits up = {&s_fail, a.patience};
     if (blockIdx.x == 0) {
         tail_cta(a, reinterpret_cast<uint8_t*>(sA), up);
         return;
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                     if (n_pieces > kRing << lg) lane_rows(unit_rows(op, m, unit), q0, q1);
 #pragma unroll 1
                     for (int c = warp & ((1 << lg) - 1); c < n_pieces; c += 1 << lg) {
-                        if (!mbar_wait(full + 8 * c_slot, c_phase)) up.now();
+                        if (!mbar_wait(full + 8 * c_slot, c_phase)) *up.failed = 1;
                         uint4 w0, w1;
                         {
                             const uint32_t src = ring + c_slot * 1024;
@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
                 else project(std::integral_constant<int, kSR>{}, m, op, epoch);
             }
             if (m == kOpQKV) {
-                if (op == 0 && step > 0 && tid == 0 && !bar.wait(600ull * a.patience)) up.now();  // the cache rows of the step before
+                if (op == 0 && step > 0 && tid == 0 && !bar.wait(600ull * a.patience)) *up.failed = 1;  // the cache rows of the step before
                 workers_sync();
 #pragma unroll 1
                 for (int it = cta; it < rows_used * d.n_heads; it += G) {
@@ -862,10 +862,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_simt_kernel(const __grid_con
             }
         }
         workers_sync();
-        if (step + 1 == a.max_steps) break;
-        if (tid == 0) bar.arrive();
+        if (tid == 0 && !*up.failed) bar.arrive();
     }
     *(volatile int*)&s_stop = 1;
+    if (tid == 0 && *up.failed) atomicExch(a.dev_err, kDevErrSteps);
 }
 
 // ---- host side -----------------------------------------------------------------------------------------------------
