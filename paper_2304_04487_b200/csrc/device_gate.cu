@@ -10,11 +10,13 @@ namespace llma {
 
 namespace {
 constexpr int kMaxDevices = 64;
+constexpr int kMostShares = 4;  // launches of whole steps side by side
 struct Gate {
     std::mutex mu;
     std::vector<GateMember*> members;
     std::condition_variable over;  // a call is
     int steppers = 0;              // members that take whole steps
+    unsigned long long turns = 0;  // of whole-step launches so far
 };
 Gate g_gates[kMaxDevices];
 bool known(int device) { return device >= 0 && device < kMaxDevices; }
@@ -82,12 +84,31 @@ void GateTurn::wait_for_others(const GateMember* self, cudaStream_t stream, int 
     }
 }
 
-GateTurn::GateTurn(GateMember& m, int kind) : m_(&m), device_(m.device), kind_(kind) {
+// The launches of other calls, newest first: those that this one does not fit beside have to be over before it begins.
+void GateTurn::share_sms(int num_sms) {
+    std::vector<const GateMember*> others;
+    int callers = 1;
+    for (const GateMember* o : g_gates[device_].members) {
+        if (o == m_ || o->stream == m_->stream || !o->in_call || !o->steps) continue;
+        ++callers;
+        if (o->launched[kTurnSteps]) others.push_back(o);
+    }
+    std::sort(others.begin(), others.end(), [](const GateMember* x, const GateMember* y) { return x->turn > y->turn; });
+    ctas_ = std::max(num_sms / callers, num_sms / kMostShares);
+    int room = num_sms - ctas_;
+    for (const GateMember* o : others) {
+        room -= o->ctas;
+        if (room < 0 && err_ == cudaSuccess) err_ = cudaStreamWaitEvent(m_->stream, o->ev[kTurnSteps], 0);
+    }
+}
+
+GateTurn::GateTurn(GateMember& m, int kind, int num_sms) : m_(&m), device_(m.device), kind_(kind), ctas_(num_sms) {
     if (kind == kTurnNone) return;
     std::unique_lock<std::mutex> lock(g_gates[device_].mu);
     if (g_gates[device_].steppers == 0) return;  // (an engine that changes this waits for the call to end)
     lock_ = std::move(lock);
     wait_for_others(m_, m.stream, kind);
+    if (kind == kTurnSteps) share_sms(num_sms);
 }
 GateTurn::GateTurn(int device, cudaStream_t stream) : device_(device), kind_(kTurnTiles) {
     if (!known(device)) return;
@@ -105,6 +126,10 @@ cudaError_t GateTurn::end() {
             if (err_ == cudaSuccess) err_ = e;
         }
         m_->launched[kind_] = true;
+        if (kind_ == kTurnSteps) {
+            m_->ctas = ctas_;
+            m_->turn = ++g_gates[device_].turns;
+        }
     }
     lock_.unlock();
     return err_;

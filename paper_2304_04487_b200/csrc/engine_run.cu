@@ -204,11 +204,13 @@ static void enqueue_step_body(llma_engine* e, int n, int k, bool plan_next) {
     enqueue_tail(e, n, k, true, plan_next);
 }
 
-// Up to `steps` decoding steps as launches of the whole-step kernel (fewer if no sequence has anything left to do), each with its plan
-static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps) {
+// Up to `steps` decoding steps as launches of the whole-step kernel on `ctas` SMs (fewer if no sequence has anything left to do), each with
+// its plan
+static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps, int ctas) {
     SimtStep s = e->simt;
     e->plain_acts = true;
     s.tail = tail_args(e, n, k);
+    s.patience = (int)std::min<int64_t>(1 << 22, (int64_t)s.patience * e->num_sms / ctas);
     const uint32_t per_step = simt_epochs(e->dims);
     for (; steps > 0; steps -= kStepsPerLaunch) {
         s.max_steps = std::min(steps, kStepsPerLaunch);
@@ -218,7 +220,7 @@ static int enqueue_whole_steps(llma_engine* e, int n, int k, int steps) {
         }
         s.epoch = e->ll_epoch;
         e->ll_epoch += per_step * (uint32_t)s.max_steps;
-        CU_TRY(launch_step_simt(e->stream, e->bf16, s, e->simt_smem, e->num_sms));
+        CU_TRY(launch_step_simt(e->stream, e->bf16, s, e->simt_smem, ctas));
         e->launch_counter += 1;
     }
     return LLMA_OK;
@@ -485,8 +487,8 @@ static int turn_kind(const llma_engine* e, bool whole) {
     return whole ? kTurnSteps : (e->gemm_impl == LLMA_GEMM_TCGEN05 ? kTurnTiles : kTurnNone);
 }
 
-static int enqueue_lone_step(llma_engine* e, int n, int k) {  // plan, forward pass, acceptance
-    if (e->step_simt) return enqueue_whole_steps(e, n, k, 1);
+static int enqueue_lone_step(llma_engine* e, int n, int k, int ctas) {  // plan, forward pass, acceptance
+    if (e->step_simt) return enqueue_whole_steps(e, n, k, 1, ctas);
     auto enqueue = [&] { enqueue_tail(e, n, k, false, true); enqueue_step_body(e, n, k, false); };
     llma_engine::StepGraph& g = graph_entry(e, e->lone_graphs, n, k);
     if (!e->can_capture || g.uses + 1 < kCaptureAt) {
@@ -535,9 +537,9 @@ extern "C" int llma_step(llma_engine* e, int32_t n, int32_t k, int32_t* out_toke
     if (rc) return rc;
     std::chrono::steady_clock::time_point gave_up{};
     for (bool again = true; again;) {
-        GateTurn turn(e->gate, turn_kind(e, e->step_simt));
+        GateTurn turn(e->gate, turn_kind(e, e->step_simt), e->num_sms);
         CU_TRY(turn.error());
-        rc = enqueue_lone_step(e, n, k);
+        rc = enqueue_lone_step(e, n, k, turn.ctas());
         if (rc) return rc;
         CU_TRY(turn.end());
         // the tokens a step can have emitted come back with the state
@@ -659,12 +661,12 @@ extern "C" int llma_generate(llma_engine* e, int32_t max_new, int32_t n, int32_t
         }
         if (left <= 0) break;
         int batch = (left + k) / (k + 1);
-        GateTurn turn(e->gate, kind);
+        GateTurn turn(e->gate, kind, e->num_sms);
         CU_TRY(turn.error());
         if (whole) {
             const int64_t before = e->launch_counter;
             const int most = shared ? kStepsPerTurn : std::max(kStepsPerLaunch, 2 * batch);
-            rc = enqueue_whole_steps(e, n, k, std::min(left, most));
+            rc = enqueue_whole_steps(e, n, k, std::min(left, most), turn.ctas());
             launches += e->launch_counter - before;
             e->launch_counter = before;
         } else {
@@ -786,10 +788,10 @@ extern "C" int llma_generate_forced(llma_engine* e, int32_t seq, const int32_t* 
         for (int at = 0; at < n_steps;) {
             const int now = std::min(n_steps - at, shared ? kStepsPerTurn : n_steps);
             if (at > 0) CU_TRY(cudaStreamSynchronize(e->stream));
-            GateTurn turn(e->gate, kind);
+            GateTurn turn(e->gate, kind, e->num_sms);
             CU_TRY(turn.error());
             e->launch_counter = before;
-            if (whole) rc = enqueue_whole_steps(e, 1, 0, now);
+            if (whole) rc = enqueue_whole_steps(e, 1, 0, now, turn.ctas());
             else rc = launch_steps(e, graph, 1, 0, now);
             if (rc) return rc;
             launches += whole ? e->launch_counter - before : (int64_t)now * e->launches_per_step;
@@ -858,7 +860,7 @@ extern "C" int llma_profile_steps(llma_engine* e, int32_t n, int32_t k, int32_t 
         if (rc) return rc;
         e->prof_on = true;
         e->prof_n = 0;
-        GateTurn turn(e->gate, turn_kind(e, false));
+        GateTurn turn(e->gate, turn_kind(e, false), e->num_sms);
         CU_TRY(turn.error());
         mark(e, -1);
         enqueue_tail(e, n, k, false, true);

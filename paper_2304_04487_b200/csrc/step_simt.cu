@@ -931,13 +931,13 @@ cudaError_t init_step_simt(bool bf16, int head_dim, size_t smem, bool* fits) {
 }
 
 template <typename T, int HD>
-static cudaError_t launch_typed(cudaStream_t st, const SimtStep& s, size_t smem, int num_sms) {
+static cudaError_t launch_typed(cudaStream_t st, const SimtStep& s, size_t smem, int ctas) {
     void* args[] = {const_cast<SimtStep*>(&s)};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(step_simt_kernel<T, HD>), dim3(num_sms), dim3(kThreads), args, smem, st);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(step_simt_kernel<T, HD>), dim3(ctas), dim3(kThreads), args, smem, st);
 }
-cudaError_t launch_step_simt(cudaStream_t st, bool bf16, const SimtStep& s, size_t smem, int num_sms) {
-    if (bf16) return s.dims.head_dim == 128 ? launch_typed<__nv_bfloat16, 128>(st, s, smem, num_sms) : launch_typed<__nv_bfloat16, 64>(st, s, smem, num_sms);
-    return s.dims.head_dim == 128 ? launch_typed<float, 128>(st, s, smem, num_sms) : launch_typed<float, 64>(st, s, smem, num_sms);
+cudaError_t launch_step_simt(cudaStream_t st, bool bf16, const SimtStep& s, size_t smem, int ctas) {
+    if (bf16) return s.dims.head_dim == 128 ? launch_typed<__nv_bfloat16, 128>(st, s, smem, ctas) : launch_typed<__nv_bfloat16, 64>(st, s, smem, ctas);
+    return s.dims.head_dim == 128 ? launch_typed<float, 128>(st, s, smem, ctas) : launch_typed<float, 64>(st, s, smem, ctas);
 }
 
 }  // namespace llma

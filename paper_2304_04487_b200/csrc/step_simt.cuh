@@ -46,6 +46,7 @@ inline size_t simt_rows_words(int row_cap) { return 2 * (2 + 4 * (size_t)row_cap
 // Whether the shape can run this way; fills geo, pass_rows, the offsets and the launch's shared memory.
 bool step_simt_shape(const ModelDims& d, bool bf16, int y_cap, int num_sms, SimtStep* s, size_t* smem);
 cudaError_t init_step_simt(bool bf16, int head_dim, size_t smem, bool* fits);
-cudaError_t launch_step_simt(cudaStream_t st, bool bf16, const SimtStep& s, size_t smem, int num_sms);
+// What a step gives does not depend on the number of CTAs (two at least).
+cudaError_t launch_step_simt(cudaStream_t st, bool bf16, const SimtStep& s, size_t smem, int ctas);
 
 }  // namespace llma
