@@ -240,10 +240,11 @@ __device__ __forceinline__ void attend(const SimtStep& a, const StepRows& R, int
         s = on ? s * scale : -INFINITY;
         float m = fmaxf(M, s);
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));  // finite: the sweep's first position is one of them
-        const float f = expf(M - m);                        // 0 at first
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        const float ref = m == -INFINITY ? 0.f : m;         // (scores that have overflowed, and nothing else so far)
+        const float f = expf(M - ref);                      // 0 at first
         M = m;
-        s = expf(s - m);  // 0 past pos
+        s = expf(s - ref);  // 0 past pos
         l = fmaf(l, f, s);
 #pragma unroll
         for (int c = 0; c < NF; ++c) o[c] *= f;

@@ -133,3 +133,25 @@ def test_launches_that_give_up_are_repeated(name):
     eng.llma_debug_set_device_error(4)
     assert generate(0) > 3                                         # those that did nothing, and those that did
     eng.llma_destroy()
+
+
+def test_positions_without_weight_come_first():
+    """Scores of minus infinity (products that overflow) at the first positions, where a warp of the attention has seen nothing else yet:
+    they weigh nothing, as they do for the oracle."""
+    from oracle import model as OM
+    from parity import step_parity
+    from paper_2304_04487_b200 import Engine
+    V, d, bad = 77, 64, 8
+    shape = ModelShape("overflow", 1, d, 1, 64, 64, V, "fp32")
+    w = make_weights(shape, seed=0, std=0.3)
+    w["tok_emb"][:, :2] = [1.0, 0.0]          # ordinary tokens: a query of 1e20 in a slow rotary pair, a key of 0
+    w["tok_emb"][:bad, :2] = [0.0, -1.0]      # the others: a query of 0, a key of -1e20
+    w["lm_head"][:bad] = 0.0
+    for name, col in (("wq.0", 0), ("wk.0", 1)):
+        w[name][31], w[name][63] = 0.0, 0.0
+        w[name][31, col] = 1e20
+    prompt = list(range(bad)) + [int(t) for t in make_prompt(7, V - bad, seed=1) + bad]
+    eng = Engine(shape, w, max_seq=64, max_ref=32, max_k=3, keep_logits=True)
+    rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=64), prompt, prompt[bad:], None, 1, 3, 20, "fp32")
+    assert np.isfinite(rep.max_logit_scale) and min(rep.tokens) >= bad and rep.near_ties == 0
+    eng.llma_destroy()
