@@ -86,7 +86,37 @@ static cudaError_t alloc_prompt_buffers(llma_engine* e) {
     return r;
 }
 
-// Whole decoding steps on the CUDA cores in one launch, where the rows of a pass fit shared memory
+// Where whole steps on the CUDA cores pay.  They save the ends of launches, some 10 us a layer, and lose where a step has many rows: a matrix
+// is read once per pass, the rows of a pass are bounded by the widest input, and their products cost more here.  Decodes alternate
+// between steps of one row a sequence and steps of all rows; the lines were drawn with references that agree with 60 and 95 % of
+// the text (a tenth to a fifth and a third to a half of the steps are copies).  Times launches / whole steps, 60 and 95 %:
+//
+// Against launches on the CUDA cores (fp32; bf16 the same), width / FFN width, rows of one or four sequences: 256 / 1024 4 x 19 1.70, 1.39;
+// 512 / 1408 4 x 19 1.35, 1.17; 1024 / 2816 16 rows in two passes 1.55, 1.16, 4 x 9 in four for three 1.14, 0.92, 4 x 19 in eight for five 1.15, 0.92;
+// 1536 / 4096 9 rows in two passes for one 1.31, 1.03, 16 in three for one 1.54, 1.08; 2048 / 5632 5 in two for one 1.19, 0.93, 9 in three for
+// one 1.26, 0.95, and where only two rows fit a pass: 2048 / 8192 5 rows 1.07, 0.77, 1024 / 8192 9 rows 1.08, 0.74, 512 / 8192 5 rows 1.20, 0.86.
+// So at least four rows have to fit, and matrices may be read twice more than by the launches at most.
+//
+// Against tensor cores, width, FFN width, vocabulary, rows, positions: 256, 1024, 4096, 16, 650 1.62, 1.42; 512, 1408, 5000, 16, 300 1.47, 1.20, at 650
+// 1.29, 1.08; vocabulary 32000, 9, 300 1.24, 1.04, 16, 650 1.16, 0.97; 128000, 5, 300 1.19, 1.05, 16, 300 1.17, 0.90; six layers 512, 2048, 32000, 16, 300 1.25,
+// 1.03, at 650 1.10, 0.92; more than a pass: 512, 4096, 5000, 9, 60 1.18, 0.89, 512, 8192, 5000, 9, 300 0.73, 0.47.  Width 1024, two layers, 13 rows,
+// 2000 positions lost a third (a row and head is one CTA's work here, 0.6 us per 64 positions).  So one pass, and the products of a layer
+// and of a part of the LM head bounded by a line that falls with the positions.
+static bool whole_steps_pay(const llma_engine* e, const SimtStep& s) {
+    const ModelDims& d = e->dims;
+    const int rows = d.max_batch * d.kp1;
+    if (e->gemm_impl != LLMA_GEMM_TCGEN05) {
+        if (s.passes > 1 && s.pass_rows < 4) return false;
+        for (int k_in : {d.d_model, d.hd_total, d.d_ffn})
+            if (s.passes > rowgemm_passes(rows, k_in) + 2) return false;
+        return true;
+    }
+    const int64_t layer = 4ll * d.d_model * d.hd_total + 3ll * d.d_model * d.d_ffn, head = (int64_t)d.d_model * d.vocab / (4 * d.n_layers);
+    return s.passes == 1 && d.d_model <= 512 && d.d_model * d.max_batch <= 1024 && d.max_seq <= 768 &&
+           rows * (layer + head) <= 190000ll * (1100 - d.max_seq);
+}
+
+// Whole decoding steps in one launch, where they are possible and pay
 static cudaError_t init_whole_steps(llma_engine* e) {
     const ModelDims& d = e->dims;
     int coop = 0;
@@ -94,7 +124,7 @@ static cudaError_t init_whole_steps(llma_engine* e) {
     if (r != cudaSuccess) return r;
     SimtStep& s = e->simt;
     bool fits = false;
-    if (!coop || !step_simt_shape(d, e->bf16, e->y_cap, e->num_sms, &s, &e->simt_smem)) return cudaSuccess;
+    if (!coop || !step_simt_shape(d, e->bf16, e->y_cap, e->num_sms, &s, &e->simt_smem) || !whole_steps_pay(e, s)) return cudaSuccess;
     r = init_step_simt(e->bf16, d.head_dim, e->simt_smem, &fits);
     if (r != cudaSuccess || !fits) return r;
     std::vector<SimtOp> ops;
@@ -348,15 +378,8 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
             if (e->prompt_pairs < 1) { free_engine(e); return LLMA_ERR_CONFIG; }
         }
     }
-    // Decoding steps of narrow decoders run whole on the CUDA cores: at these widths a step costs the ends of its launches, not its
-    // weights.  The line lies where the two cost the same.  us per decode, launches of tensor-core kernels -> whole steps: width 256, two
-    // layers, up to 16 rows at 700 positions 1202 -> 844, four sequences 1834 -> 1359; width 512, three layers, up to six rows, a call per
-    // step 1536 -> 1335, up to 16 rows at 700 positions 1649 -> 1404, two sequences 1837 -> 1779, four 2409 -> 2438; width 1024, two
-    // layers, up to nine rows at 600 positions 1987 -> 1965, up to thirteen at 2000 positions 1993 -> 2672 (a row and head is one CTA's
-    // work here, 0.6 us per 64 positions).  All rows in one pass; an engine asked for the tensor cores keeps to them.
-    if (e->gemm_impl == LLMA_GEMM_TCGEN05 && cfg->gemm_impl == LLMA_GEMM_AUTO && e->decode_rows <= 16 && d.d_model <= 512 &&
-        d.d_model * d.max_batch <= 1024 && d.max_seq <= 768)
-        CREATE_TRY(init_whole_steps(e));
+    // (an engine asked for the tensor cores keeps to them)
+    if (e->gemm_impl == LLMA_GEMM_TCGEN05 && cfg->gemm_impl == LLMA_GEMM_AUTO) CREATE_TRY(init_whole_steps(e));
     {
         // page-locked memory in one piece: every such allocation costs about a millisecond
         size_t total = 0;

@@ -72,6 +72,8 @@ struct RowGemm {
 cudaError_t init_rowgemm(bool bf16);
 // row_bound: most rows of a step (more than a pass takes: further passes over the weights inside the launch)
 void launch_rowgemm(cudaStream_t st, bool bf16, RowGemm g, int row_bound, int num_sms);
+// passes over a matrix with inputs of this width
+int rowgemm_passes(int rows, int k_in);
 // CTAs of a launch (the number of partial maxima of kRowHead)
 int rowgemm_grid(int n_units, int k_in, int row_bound, int num_sms);
 // causal attention of every used row over its sequence's cache rows [0, pos]; n_rows = the row slots of the pass

@@ -332,6 +332,10 @@ static int pass_rows_of(int row_bound, int k_in) {
     const int passes = (rows + most - 1) / most;
     return ((rows + passes - 1) / passes + 3) / 4 * 4;
 }
+int rowgemm_passes(int rows, int k_in) {
+    const int each = pass_rows_of(rows, k_in);
+    return (rows + each - 1) / each;
+}
 static bool is_resident(int pass_rows, int k_in) { return (size_t)pass_rows * k_in * sizeof(float) <= kResidentBytes; }
 static int cta_cap(int k_in, int pass_rows, int num_sms) {  // CTAs that the GPU holds at once
     return num_sms * (is_resident(2 * pass_rows, k_in) ? 2 : 1);

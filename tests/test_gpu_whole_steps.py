@@ -155,3 +155,28 @@ def test_positions_without_weight_come_first():
     rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=64), prompt, prompt[bad:], None, 1, 3, 20, "fp32")
     assert np.isfinite(rep.max_logit_scale) and min(rep.tokens) >= bad and rep.near_ties == 0
     eng.llma_destroy()
+
+
+@pytest.mark.parametrize("whole,d,heads,hd,ffn,vocab,dtype,k,B,max_seq", [
+    (True, 256, 4, 64, 1024, 515, "fp32", 18, 4, 96),        # 76 rows: five passes either way
+    (True, 320, 5, 64, 4096, 301, "fp32", 15, 1, 96),        # 16 rows: three passes of six, the launches two of eight
+    (False, 320, 5, 64, 8192, 301, "fp32", 4, 1, 96),        # two rows a pass
+    (False, 320, 5, 64, 4096, 301, "fp32", 8, 4, 96),        # 36 rows: six passes for three
+    (True, 320, 5, 64, 8192, 301, "fp32", 1, 1, 96),         # two rows, one pass
+    (True, 512, 8, 64, 2048, 301, "bf16", 15, 1, 96), (False, 512, 8, 64, 2048, 301, "bf16", 15, 1, 768),   # the line of positions
+    (True, 512, 8, 64, 2048, 301, "bf16", 7, 1, 768), (False, 512, 8, 64, 2048, 301, "bf16", 7, 1, 769),
+    (False, 512, 8, 64, 4096, 301, "bf16", 8, 1, 96), (True, 512, 8, 64, 4096, 301, "bf16", 4, 1, 96),      # more than a pass; one
+    (False, 512, 4, 64, 512, 60000, "bf16", 15, 1, 600), (True, 512, 4, 64, 512, 60000, "bf16", 7, 1, 600)])  # the LM head's share
+def test_whole_steps_where_they_pay(whole, d, heads, hd, ffn, vocab, dtype, k, B, max_seq):
+    from paper_2304_04487_b200 import Engine
+    shape = ModelShape(f"pay-{d}-{ffn}", 1, d, heads, hd, ffn, vocab, dtype)
+    eng = Engine(shape, make_weights(shape, seed=0, std=0.05), max_seq=max_seq, max_ref=64, max_k=k, max_batch=B)
+    for s in range(B):
+        eng.llma_prefill(s, make_prompt(20 + s, vocab, seed=s))
+    greedy, st = eng.llma_generate(20, 1, 0)
+    assert (st.launches == 1) == whole
+    for s in range(B):
+        eng.llma_set_reference(s, greedy[s])
+        eng.llma_rewind(s)
+    assert eng.llma_generate(20, 1, k)[0] == greedy
+    eng.llma_destroy()
