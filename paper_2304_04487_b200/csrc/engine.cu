@@ -139,7 +139,13 @@ static cudaError_t init_whole_steps(llma_engine* e) {
     e->ll_count = rc * (d.d_model + 4 * (size_t)d.hd_total + d.d_ffn) + parts + simt_rows_words(e->row_cap);
     // one block: the words, the barrier's, the ops
     const size_t words = e->ll_count + 1 + (ops.size() * sizeof(SimtOp) + 7) / 8;
-    if ((r = dalloc(&e->ll_words, words)) != cudaSuccess) return r;
+    r = dalloc(&e->ll_words, words);
+    if (r == cudaErrorMemoryAllocation) {  // no room for them: steps are launched kernel by kernel, which needs none
+        cudaGetLastError();
+        e->ll_words = nullptr;
+        return cudaSuccess;
+    }
+    if (r != cudaSuccess) return r;
     e->grid_barrier = reinterpret_cast<uint32_t*>(e->ll_words + e->ll_count);
     SimtOp* step_ops = reinterpret_cast<SimtOp*>(e->ll_words + e->ll_count + 1);
     if ((r = cudaMemcpy(step_ops, ops.data(), ops.size() * sizeof(SimtOp), cudaMemcpyHostToDevice)) != cudaSuccess) return r;

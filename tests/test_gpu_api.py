@@ -260,3 +260,37 @@ assert all(np.array_equal(x, y) for x, y in zip(rows(c), want))
 """
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
+
+
+def test_whole_steps_do_without_where_memory_is_short():
+    """An engine for whose whole steps there is no room launches its steps kernel by kernel instead of failing: the same tokens.  (In a
+    process of its own, which takes all but part of the memory that the engine would like to have.)"""
+    import os
+    import subprocess
+    import sys
+    code = """
+import torch
+from paper_2304_04487_b200 import Engine
+from workloads import ModelShape, make_prompt, make_weights
+shape = ModelShape("words", 1, 1024, 8, 128, 2048, 300, "fp32")
+kw = dict(max_seq=40, max_ref=8, max_k=7, max_batch=32)                 # 256 rows: 16 MB of words
+a = Engine(shape, make_weights(shape, seed=0), **kw)
+prompt = make_prompt(9, shape.vocab, seed=3)
+free = lambda: (torch.cuda.synchronize(), torch.cuda.mem_get_info()[0])[1]
+def decode(eng):
+    eng.llma_prefill(0, prompt)
+    (y,), st = (lambda t, s: (t[:1], s))(*eng.llma_generate(6, 1, 0))
+    return y, st.launches
+want, launches = decode(a)
+assert launches == 1
+before = free()
+b = Engine(shape, None, share_weights_with=a, **kw)
+size = before - free()
+b.llma_destroy()
+taken = torch.empty(free() - (size - (8 << 20)), dtype=torch.uint8, device="cuda")
+c = Engine(shape, None, share_weights_with=a, **kw)
+got, launches = decode(c)
+assert got == want and launches > 6
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
