@@ -579,7 +579,8 @@ def main():
             eng.llma_rewind(0)
             _, st = eng.llma_generate(n_new, n, k)
             tot += st.launches
-        print(json.dumps({"profile_only": True, "launches_per_step": g0.launches // n_new,
+        # (less than one where a launch takes many steps)
+        print(json.dumps({"profile_only": True, "launches_per_step": max(g0.launches // n_new, round(g0.launches / n_new, 3)),
                           "greedy_launches": int(g0.launches), "llma_launches": int(tot),
                           "llma_steps": int(st.steps), "llma_ms_per_step": st.device_ms / st.steps}))
         return
@@ -661,6 +662,11 @@ def main():
                 "per_class": per_class_roofline(shape, prof, kvbytes, peak),
                 "per_class_note": "launched one by one with an event after every kernel (no overlap between "
                                   "kernels): each class's rate inside the graph is at least this"}
+    if g0.launches < n_new:                              # whole steps: one kernel, none of those profiled above
+        whole = roofline["whole_step"]
+        roofline = {"bound": "hbm", "kernel": "step_simt_kernel", "achieved": whole["frac"] * peak, "peak": peak, "unit": "GB/s",
+                    "frac": whole["frac"], "peak_kind": f"of {peak_kind}", "traffic": None, "launches_per_step": g0.launches / n_new,
+                    "whole_step": whole}
 
     # step latency against k: reference = y* itself, so every step feeds k+1 rows.  k <= 8 on the
     # benchmark's engine (16-row MMA shape); k = 16 needs an engine created for 17 rows (32-row shape)

@@ -64,7 +64,8 @@ typedef struct {
     float rms_eps;        /* RMSNorm epsilon */
     float rope_theta;     /* rotary base; pairing is (i, i + head_dim/2) */
     int32_t eos_id;       /* -1: none.  Otherwise a sequence stops after emitting this id */
-    int32_t gemm_impl;    /* LLMA_GEMM_*; AUTO = tensor-core kernels for bf16, SIMT for fp32 */
+    int32_t gemm_impl;    /* LLMA_GEMM_*; AUTO = SIMT for fp32, tensor-core kernels for bf16, except that decoding steps of narrow decoders
+                             (d_model <= 512, a few rows, short contexts) run on the CUDA cores, whole steps in one launch */
     int32_t keep_logits;  /* 1: keep the last step's logits for llma_debug_logits */
 } llma_config;
 
@@ -109,7 +110,9 @@ typedef struct {
  * Create an engine on the current CUDA device.  `cuda_stream` is a cudaStream_t (may be
  * NULL for the default stream, where steps are launched kernel by kernel because CUDA does not capture it;
  * on any other stream they run as graphs, kept for the last 64 (n, k) and captured by llma_generate at once, by
- * llma_step from the sixteenth use on); all work of the engine is issued on it.  Allocates the K/V
+ * llma_step from the sixteenth use on); all work of the engine is issued on it.  Decoding steps on the CUDA cores run
+ * whole, up to 32 of them in one launch without a graph, wherever that pays.  Engines on streams of their own may be used
+ * side by side, each by one thread at a time; launches of whole steps and of tensor-core projections take turns.  Allocates the K/V
  * cache ([layer][seq][head][max_seq][head_dim], zero-filled), reference storage and
  * workspaces, among them, on the tensor-core path, 4 * (2 d_model + 2 n_heads*head_dim + d_ffn) bytes for each position of a
  * prompt pass (up to 2048 positions, 224 MB at the 7B widths; fewer positions, down to 128, where memory is short), and
@@ -283,10 +286,12 @@ typedef struct {
 } llma_profile;
 
 /*
- * Measurement aid: run `steps` decoding steps exactly like llma_step (state advances, tokens
+ * Measurement aid: run `steps` decoding steps like llma_step (state advances, tokens
  * are appended) but with a CUDA event recorded on the engine's stream after every kernel
  * launch; the time between consecutive events is attributed to the kernel just launched.
  * Launches are direct (no graph), so the figures include the gap to the previous kernel.
+ * Engines whose steps run whole in one launch take these through the kernels that such a launch stands in for: another
+ * order of sums, and figures of kernels that their llma_step does not run.
  * Errors: as llma_step.
  */
 int llma_profile_steps(llma_engine *e, int32_t n, int32_t k, int32_t steps, llma_profile *out);
@@ -336,14 +341,15 @@ int llma_gemm_rows32_bf16(const void *W, const void *a, float *out, int32_t n_ou
  * error words.  All calls on a device share the array and it keeps the previous call's contents: a call leaves the
  * hand-over slots empty, and empties them first if the call before did not end well, but two calls that overlap on
  * the GPU (different streams, or different threads) race on it and give wrong results -- serialise them.  The call is
- * synchronous: it waits for the kernel and looks at its error word before it returns.
+ * synchronous: it waits for the kernel and looks at its error word before it returns.  What it keeps does not outlive the device's
+ * context: no calls after a cudaDeviceReset.
  * Errors: NULL, ARG, CAPACITY, CONFIG (not an sm_100 device), CUDA, DEVICE_TIMEOUT.
  */
 int llma_gemm_rows32_bf16_noalloc(const void *W, const void *a, float *out, int32_t n_out, int32_t k_in,
                                   void *cuda_stream);
 
 /* Which GEMM implementation the engine resolved to (LLMA_GEMM_SIMT or LLMA_GEMM_TCGEN05), or a
- * negative status. */
+ * negative status.  An engine of the latter may still run its decoding steps on the CUDA cores (see gemm_impl). */
 int llma_gemm_impl(llma_engine *e);
 
 /* The CUDA error code behind the most recent LLMA_ERR_CUDA on this thread (0 if none). */

@@ -1,5 +1,6 @@
-// A barrier over all CTAs of a cooperative launch, one word of global memory: CTA 0 adds 2^31 - (CTAs - 1), every other CTA 1, so the
-// top bit flips when the last one has arrived and the word is ready for the next round (and the next launch) as it is.
+// A barrier over all CTAs of a cooperative launch, one word of global memory, by the scheme of the grid barrier in CUDA's cooperative
+// groups, split into arrival and wait: CTA 0 adds 2^31 - (CTAs - 1), every other CTA 1, so the top bit flips when the last one has
+// arrived and the word is ready for the next round (and the next launch, of as many CTAs as it likes) as it is.
 //
 // arrive / wait are called by ONE thread, between barriers of its CTA: what the CTA's other threads wrote before the first of these
 // is visible to every thread of every CTA after the second one (release and acquire at GPU scope, which cover them).

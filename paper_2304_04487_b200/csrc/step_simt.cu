@@ -1,5 +1,5 @@
-// Whole decoding steps on the CUDA cores (fp32 models, the cross-check of the tensor-core path, and narrow bf16 decoders: the rule and
-// what it measured are in engine.cu) in one cooperative launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
+// Whole decoding steps on the CUDA cores (decoders of the CUDA-core path and narrow bf16 decoders, where that pays: the rule and what it
+// measured are in engine.cu) in one cooperative launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
 //
 // At the widths this path serves a step is a chain of short phases and costs their latency.  As launches of their own
 // (kernels_simt.cu, attention_simt.cu) a phase is released about 1 us after its predecessor has ended, fetches its rows, and runs
@@ -8,10 +8,11 @@
 // that wrote it, and a reader polls the words themselves: one trip to L2 each way.  A word is written again only by a CTA that has
 // seen a result of every reader of its old value (a projection's results depend on all of its rows' values), so there is nothing to
 // clear and nothing to wait for.  One grid barrier per step makes the step's cache rows visible to the next one (the step itself takes
-// its own K/V rows from the words); it is passed while the next step's first projection runs.
+// its own K/V rows from the words); it is passed while the next step's first projection runs, and the last one stands before the state is
+// written back.
 //
-// CTA 0 does acceptance and plan, with states, references and emitted tokens in its shared memory.  The others, one per SM, sixteen
-// warps each, do everything else.  A warp takes four pairs of output features (of a rotary pair, of gate and up, of neighbours):
+// CTA 0 does acceptance and plan, with states, references and emitted tokens in its shared memory.  The others, one per SM (of all, or of
+// a share of them: device_gate.h), sixteen warps each, do everything else.  A warp takes four pairs of output features (of a rotary pair, of gate and up, of neighbours):
 // eight lanes per pair, each with its own columns of the two weight rows, all rows' sums in registers, the rows themselves in
 // shared memory, where a warp's access is one 128-byte line; 2 to 16 warps share the columns of a unit.  Units are dealt over the SMs
 // first, so that every SM pulls weights whatever the width.  Weights come through a ring of four pieces per warp: four more warps
@@ -899,11 +900,10 @@ bool step_simt_shape(const ModelDims& d, bool bf16, int y_cap, int num_sms, Simt
     if (*smem < tail) *smem = (tail + 15) / 16 * 16;
     if (*smem > kStepSmem) return false;
     const int pairs[5] = {3 * d.hd_total / 2, d.d_model / 2, d.d_ffn, d.d_model / 2, (d.vocab + 1) / 2};
-    const int outs[5] = {3 * d.hd_total, d.d_model, d.d_ffn, d.d_model, d.vocab};
     const int ks[5] = {d.d_model, d.hd_total, d.d_model, d.d_ffn, d.d_model};
     for (int m = 0; m < 5; ++m) {
         SimtGeo& g = s->geo[m];
-        g.n_units = (pairs[m] + 3) / 4; g.n_out = outs[m]; g.k_in = ks[m];
+        g.n_units = (pairs[m] + 3) / 4; g.k_in = ks[m];
         g.n_pieces = ks[m] / (bf16 ? 64 : 32);
         g.sweep_rows = kSweep / ks[m]; g.sweep_cols = kSweep % ks[m];
         // Warps per unit: the fewest pieces in a row, counting a round of units as two pieces more

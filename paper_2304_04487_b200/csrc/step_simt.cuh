@@ -11,7 +11,7 @@ struct SimtOp {
 };
 struct SimtGeo {         // shape of a class of projections (QKV, output, gate/up, down, LM head)
     int32_t n_units;     // groups of four pairs of output features
-    int32_t n_out, k_in;
+    int32_t k_in;
     int32_t n_pieces;    // pieces of eight 16-byte loads that a weight row consists of
     int32_t split_lg;    // log2 of the warps that share a unit
     int32_t sweep_rows, sweep_cols;  // 2 * threads activations, as rows and columns of this width

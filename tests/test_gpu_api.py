@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from workloads import SHAPES, make_prompt, make_weights
+from workloads import SHAPES, ModelShape, make_prompt, make_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -115,22 +115,27 @@ def test_microbench_mma_runs_and_rejects_bad_arguments():
             llma_microbench_mma(*bad)
 
 
-@pytest.mark.parametrize("name", ["tiny-fp32", "tiny-bf16"])
-def test_engine_on_the_default_stream(setup, name):
+# shapes whose steps are launched kernel by kernel: tensor cores on request, and CUDA cores where two rows fit a pass
+LAUNCHED = {"tiny-bf16": (SHAPES["tiny-bf16"], 2), "fp32-launched": (ModelShape("fp32-launched", 2, 128, 2, 64, 8192, 515, "fp32"), 0)}
+
+
+@pytest.mark.parametrize("name,launched", [("tiny-fp32", False), ("tiny-bf16", False), ("tiny-bf16", True), ("fp32-launched", True)])
+def test_engine_on_the_default_stream(setup, name, launched):
     """cuda_stream = NULL: CUDA does not capture the legacy default stream, so every entry point has to do without graphs.
     Same tokens as on a stream of its own, whether a step is launched directly or replayed."""
     import torch
     Engine = setup[0]
-    shape = SHAPES[name]
+    shape, impl = LAUNCHED[name] if launched else (SHAPES[name], 0)
     w = make_weights(shape, seed=0)
     prompt = make_prompt(20, shape.vocab, seed=1)
-    own = Engine(shape, w, max_seq=96, max_ref=64, max_k=4)
-    null = Engine(shape, w, max_seq=96, max_ref=64, max_k=4, stream=torch.cuda.default_stream())
+    own = Engine(shape, w, max_seq=96, max_ref=64, max_k=4, gemm_impl=impl)
+    null = Engine(shape, w, max_seq=96, max_ref=64, max_k=4, gemm_impl=impl, stream=torch.cuda.default_stream())
     assert null.stream.cuda_stream == 0
     out = []
     for eng in (own, null):
         eng.llma_prefill(0, prompt)
         (y,), st = eng.llma_generate(24, 1, 0)
+        assert (st.launches > 24) == launched
         eng.llma_set_reference(0, y)
         for _ in range(5):                     # 25 steps: launched directly, captured, replayed
             steps = []
@@ -147,12 +152,18 @@ def test_engine_on_the_default_stream(setup, name):
     assert out[0][2] == out[0][0] and out[0][1] == out[0][0][:len(out[0][1])]
 
 
-def test_more_step_shapes_than_graphs_are_kept(setup):
+@pytest.mark.parametrize("name", ["tiny-fp32", *LAUNCHED])   # whole steps, which make no graphs; launches
+def test_more_step_shapes_than_graphs_are_kept(setup, name):
     """Captured steps are kept for the last 64 (n, k); one that has made room for another is captured again."""
     Engine, shape, w = setup
-    eng = Engine(shape, w, max_seq=64, max_ref=32, max_k=4)
+    impl = 0
+    if name in LAUNCHED:
+        shape, impl = LAUNCHED[name]
+        w = make_weights(shape, seed=0)
+    eng = Engine(shape, w, max_seq=64, max_ref=32, max_k=4, gemm_impl=impl)
     eng.llma_prefill(0, make_prompt(20, shape.vocab, seed=1))
-    (y,), _ = eng.llma_generate(12, 1, 0)
+    (y,), st = eng.llma_generate(12, 1, 0)
+    assert (st.launches > 12) == (name in LAUNCHED)
     eng.llma_set_reference(0, y)
     for turn in range(3):
         for n in range(1, 71):

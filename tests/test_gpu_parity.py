@@ -49,26 +49,29 @@ def test_tiny_fp32_stepwise_parity():
     assert rep.max_logit_err <= 1e-4 * max(1.0, rep.max_logit_scale)
 
 
-@pytest.mark.parametrize("name,n,k,P,N", [("tiny-bf16", 1, 8, 70, 48), ("small-bf16", 1, 5, 45, 40),
-                                           ("small-bf16", 2, 16, 33, 40), ("mid-bf16", 1, 8, 50, 32),
-                                           # contexts spanning several 128-position attention chunks with a ragged tail
-                                           ("tiny-bf16", 1, 8, 300, 24), ("small-bf16", 1, 20, 250, 30)])
-def test_bf16_stepwise_parity(name, n, k, P, N):
+# impl 0: small steps of the narrow ones are whole steps on the CUDA cores (prompts by tensor cores); 2: tensor cores throughout
+@pytest.mark.parametrize("name,n,k,P,N,impl", [("tiny-bf16", 1, 8, 70, 48, 0), ("small-bf16", 1, 5, 45, 40, 0),
+                                               ("small-bf16", 2, 16, 33, 40, 0), ("mid-bf16", 1, 8, 50, 32, 0),
+                                               # contexts spanning several 128-position attention chunks with a ragged tail
+                                               ("tiny-bf16", 1, 8, 300, 24, 0), ("small-bf16", 1, 20, 250, 30, 0),
+                                               ("tiny-bf16", 1, 8, 70, 48, 2), ("small-bf16", 1, 5, 45, 40, 2), ("tiny-bf16", 1, 8, 300, 24, 2)])
+def test_bf16_stepwise_parity(name, n, k, P, N, impl):
     shape = SHAPES[name]
     w = _weights(shape)
     prompt = make_prompt(P, shape.vocab, seed=2)
     max_seq = P + N + 40
     y_star = _greedy_star(shape, w, prompt, N, max_seq)
     ref, offs, _ = build_reference(y_star, [60, 60, 40], 0.7, shape.vocab, seed=1)
-    eng = _engine(shape, w, max_seq=max_seq, max_ref=200, max_k=k, keep_logits=True)
-    assert eng.llma_gemm_impl() == 2                     # bf16 shapes run the tensor-core GEMMs
+    eng = _engine(shape, w, max_seq=max_seq, max_ref=200, max_k=k, keep_logits=True, gemm_impl=impl)
+    assert eng.llma_gemm_impl() == 2                     # bf16 shapes run the tensor-core GEMMs (their prompts at least)
     rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=max_seq), prompt, ref, offs, n, k, N, "bf16")
     assert rep.max_logit_err <= 2e-2
     assert rep.near_ties <= 3, rep.near_ties
     assert rep.trigger_steps > 0
 
 
-def test_bf16_parity_with_prescribed_cache_codes():
+@pytest.mark.parametrize("impl", [0, 2])                 # whole steps, tensor-core launches
+def test_bf16_parity_with_prescribed_cache_codes(impl):
     """The same comparison with the cache's quantisation decisions taken alike on both sides: every code the engine
     stored must be the rounding of a value within 1e-4 of the row scale of the oracle's unrounded value, differing
     codes must be rare, and the logits then agree far inside the tolerance."""
@@ -79,7 +82,7 @@ def test_bf16_parity_with_prescribed_cache_codes():
     max_seq = P + N + 40
     y_star = _greedy_star(shape, w, prompt, N, max_seq)
     ref, offs, _ = build_reference(y_star, [60, 60, 40], 0.7, shape.vocab, seed=1)
-    eng = _engine(shape, w, max_seq=max_seq, max_ref=200, max_k=k, keep_logits=True)
+    eng = _engine(shape, w, max_seq=max_seq, max_ref=200, max_k=k, keep_logits=True, gemm_impl=impl)
     rep = step_parity(eng, OM.OracleModel(shape, w, max_seq=max_seq), prompt, ref, offs, 1, k, N, "bf16",
                       prescribe_kv=True)
     assert rep.code_violations == 0 and rep.codes_seen > 100000
@@ -187,18 +190,19 @@ def test_kv_rows_match_oracle():
                 assert np.abs(got - want).max() <= 2.0 ** -7 * max(1e-3, np.abs(want).max())
 
 
-def test_two_sequences_ragged():
+@pytest.mark.parametrize("impl", [0, 2])                 # whole steps, tensor-core launches
+def test_two_sequences_ragged(impl):
     shape = SHAPES["tiny-bf16"]
     w = _weights(shape)
     N, max_seq = 40, 128
     prompts = [make_prompt(30, shape.vocab, seed=7), make_prompt(51, shape.vocab, seed=8)]
     singles = []
     for p in prompts:
-        e1 = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=7)
+        e1 = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=7, gemm_impl=impl)
         e1.llma_prefill(0, p)
         (t,), _ = e1.llma_generate(N, 1, 0)
         singles.append(t)
-    eng = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=7, max_batch=2)
+    eng = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=7, max_batch=2, gemm_impl=impl)
     for s, p in enumerate(prompts):
         eng.llma_prefill(s, p)
     eng.llma_set_reference(0, singles[0][4:30], None)
@@ -342,7 +346,8 @@ def test_batched_generate_equals_single_sequence_runs():
     eng.llma_destroy()
 
 
-def test_device_timeout_is_reported_and_engine_recovers():
+@pytest.mark.parametrize("impl", [0, 2])                 # whole steps, tensor-core launches
+def test_device_timeout_is_reported_and_engine_recovers(impl):
     """A kernel whose bounded wait ran out leaves a code in the device error word; here the word is preset
     through the debug hook (no wait is made to run out on the GPU).  The step must report it, and the steps
     after it must be those of an undisturbed run."""
@@ -350,7 +355,7 @@ def test_device_timeout_is_reported_and_engine_recovers():
     shape = SHAPES["tiny-bf16"]
     w = _weights(shape)
     prompt = make_prompt(30, shape.vocab, seed=50)
-    eng = _engine(shape, w, max_seq=96, max_ref=8, max_k=4)
+    eng = _engine(shape, w, max_seq=96, max_ref=8, max_k=4, gemm_impl=impl)
     eng.llma_prefill(0, prompt)
     (want,), _ = eng.llma_generate(6, 1, 0)
     eng.llma_rewind(0)
@@ -371,16 +376,19 @@ def test_device_timeout_is_reported_and_engine_recovers():
     eng.llma_destroy()
 
 
-@pytest.mark.parametrize("name", ["tiny-bf16", "tiny-fp32"])
-def test_forced_replay_follows_algorithm2_trace(name):
+FP32_LAUNCHED = ModelShape("fp32-launched", 2, 128, 2, 64, 8192, 515, "fp32")   # two rows fit a pass: launches, as graphs
+
+
+@pytest.mark.parametrize("name,impl", [("tiny-bf16", 0), ("tiny-fp32", 0), ("tiny-bf16", 2), ("fp32-launched", 0)])
+def test_forced_replay_follows_algorithm2_trace(name, impl):
     """Section 3.2's measurement device: the engine is driven along the (inputs, outputs) sequence that
     Algorithm 2 derives from a target text and the references, and must reproduce the target with exactly
     those steps; the K/V rows it leaves behind are real, so ordinary decoding can go on afterwards."""
-    shape = SHAPES[name]
+    shape = FP32_LAUNCHED if name == FP32_LAUNCHED.name else SHAPES[name]
     w = _weights(shape)
     prompt = make_prompt(33, shape.vocab, seed=60)
     N, k, max_seq = 48, 6, 128
-    eng = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=k)
+    eng = _engine(shape, w, max_seq=max_seq, max_ref=128, max_k=k, gemm_impl=impl)
     eng.llma_prefill(0, prompt)
     (y_star,), _ = eng.llma_generate(N + 5, 1, 0)
     ref, offs, _ = build_reference(y_star[:N], [60, 60], 0.7, shape.vocab, seed=3)
@@ -389,6 +397,7 @@ def test_forced_replay_follows_algorithm2_trace(name):
     eng.llma_rewind(0)
     st = eng.llma_generate_forced(0, trace, y_star[:N])
     assert st.steps == len(trace) and st.tokens == N and st.copied_accepted == N - len(trace)
+    assert (st.launches > len(trace)) == (impl == 2 or shape is FP32_LAUNCHED)
     assert eng.llma_kv_len(0) == len(prompt) - 1 + N
     # the cache now holds the target's rows: greedy decoding continues with the engine's own next tokens
     (more,), _ = eng.llma_generate(5, 1, 0)
@@ -576,3 +585,39 @@ def test_prompt_codes_at_7b_widths():
     (64, 12864, "fp32", 18)])                    # beyond: chunk by chunk, 16 and 3 rows
 def test_cuda_core_rows_per_pass(d, ffn, dtype, k):
     test_cuda_core_widths(d, 1, 64, ffn, 301, dtype, k, 1)
+
+
+# ---- the launches of CUDA-core decoding steps, which engines that take whole steps keep for llma_profile_steps --------------------
+@pytest.mark.parametrize("d,heads,hd,ffn,vocab,dtype,k,B", [
+    (64, 1, 64, 64, 77, "fp32", 3, 1), (576, 9, 64, 1600, 515, "fp32", 15, 1), (576, 9, 64, 3392, 1000, "fp32", 32, 1),
+    (192, 3, 64, 448, 301, "bf16", 4, 3), (3264, 1, 64, 192, 301, "fp32", 16, 1), (256, 1, 64, 3264, 301, "bf16", 23, 1),
+    (256, 1, 64, 5184, 301, "fp32", 8, 1), (256, 1, 64, 6464, 301, "fp32", 4, 1)])
+def test_cuda_core_launches(d, heads, hd, ffn, vocab, dtype, k, B):
+    """Steps launched kernel by kernel beside whole steps of the same decoder (which the tests above compare with the oracle):
+    the same plans and acceptances, logits within the tolerance of either against the oracle."""
+    shape = ModelShape(f"odd-{d}-{ffn}-{dtype}", 2, d, heads, hd, ffn, vocab, dtype)
+    w = _weights(shape)
+    P, N = 40, 12
+    a, b = (_engine(shape, w, max_seq=P + N + k + 8, max_ref=64, max_k=k, max_batch=B, keep_logits=True) for _ in range(2))
+    for eng in (a, b):
+        for s in range(B):
+            eng.llma_prefill(s, make_prompt(P - 3 * s, vocab, seed=20 + s))
+    ys, st = a.llma_generate(N, 1, 0)
+    assert st.launches == 1                                  # whole steps
+    for eng in (a, b):
+        for s in range(B):
+            eng.llma_set_reference(s, ys[s])
+            eng.llma_rewind(s)
+    got = [0] * B
+    while min(got) < N - 2:
+        toks = a.llma_step(1, k)
+        assert b.llma_profile_steps(1, k, 1)["_total"]["launches_per_step"] == 4 + 5 * shape.n_layers
+        ia, ib = a.llma_last_step_info(), b.llma_last_step_info()
+        la, lb = a.llma_debug_logits(), b.llma_debug_logits()
+        for s in range(B):
+            assert [getattr(ia[s], f) for f in ("pos", "k_eff", "accepted", "emitted")] == [getattr(ib[s], f) for f in ("pos", "k_eff", "accepted", "emitted")]
+            rows = slice(s * (k + 1), s * (k + 1) + ia[s].k_eff + 1)
+            tol = 2e-4 * max(1.0, float(np.abs(la[rows]).max())) if dtype == "fp32" else 2 * BF16_LOGIT_TOL   # either side's own tolerance
+            assert np.abs(la[rows] - lb[rows]).max() <= tol
+            got[s] += len(toks[s])
+    a.llma_destroy(); b.llma_destroy()
