@@ -155,7 +155,17 @@ static cudaError_t init_whole_steps(llma_engine* e) {
     s.x = e->x; s.qkv = e->qkv; s.attn = (float*)e->attn; s.h = (float*)e->h; s.logits = e->cfg.keep_logits ? e->logits : nullptr;
     s.kcache = e->kcache; s.vcache = e->vcache; s.rope_cos = e->rope_cos; s.rope_sin = e->rope_sin;
     s.barrier = e->grid_barrier; s.dev_err = e->dev_err;
-    e->step_simt = true;
+    // A launch that does nothing: a stream that has only some of the SMs (a green context's) refuses one that needs them all
+    const int32_t off = kDevErrSteps, none = kDevErrNone;
+    SimtStep trial = s;
+    trial.tail.st = e->seq_state;
+    if ((r = cudaMemcpy(e->dev_err, &off, sizeof(off), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
+    if ((r = cudaDeviceSynchronize()) != cudaSuccess) return r;
+    const cudaError_t refused = launch_step_simt(e->stream, e->bf16, trial, e->simt_smem, e->num_sms);
+    if ((r = cudaStreamSynchronize(e->stream)) != cudaSuccess) return r;
+    if ((r = cudaMemcpy(e->dev_err, &none, sizeof(none), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
+    cudaGetLastError();
+    e->step_simt = refused == cudaSuccess;
     return cudaSuccess;
 }
 

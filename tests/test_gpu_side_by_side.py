@@ -84,3 +84,35 @@ def test_whole_steps_beside_other_engines(whole, tiles):
     assert not failed and min(done) > 0, (failed, done)
     for e in (a, b, c):
         e.llma_destroy()
+
+
+def test_stream_that_has_part_of_the_sms():
+    """An engine on a stream of a green context, which has 64 SMs: a launch that needs every SM is refused there, so steps are launched
+    kernel by kernel.  The same tokens."""
+    import torch
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        assert r[0] == driver.CUresult.CUDA_SUCCESS, r
+        return r[1] if len(r) == 2 else r[1:]
+    torch.zeros(1, device="cuda")
+    dev = ok(driver.cuDeviceGet(0))
+    sms = ok(driver.cuDeviceGetDevResource(dev, driver.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    groups, _, _ = ok(driver.cuDevSmResourceSplitByCount(1, sms, 0, 64))
+    green = ok(driver.cuGreenCtxCreate(ok(driver.cuDevResourceGenerateDesc([groups[0]], 1)), dev, driver.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    part = torch.cuda.ExternalStream(int(ok(driver.cuGreenCtxStreamCreate(green, driver.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))))
+    from paper_2304_04487_b200 import Engine
+    shape = SHAPES["tiny-fp32"]
+    w = make_weights(shape, seed=0)
+    got = []
+    for stream in (None, part):
+        eng = Engine(shape, w, max_seq=96, max_ref=64, max_k=4, stream=stream)
+        eng.llma_prefill(0, make_prompt(20, shape.vocab, seed=1))
+        (y,), st = eng.llma_generate(24, 1, 0)
+        eng.llma_set_reference(0, y)
+        eng.llma_rewind(0)
+        assert eng.llma_generate(24, 1, 4)[0][0] == y
+        got.append(y)
+        assert (st.launches == 1) == (stream is None)
+        eng.llma_destroy()
+    assert got[0] == got[1]
