@@ -580,7 +580,7 @@ def main():
             _, st = eng.llma_generate(n_new, n, k)
             tot += st.launches
         # (less than one where a launch takes many steps)
-        print(json.dumps({"profile_only": True, "launches_per_step": max(g0.launches // n_new, round(g0.launches / n_new, 3)),
+        print(json.dumps({"profile_only": True, "launches_per_step": g0.launches // n_new or round(g0.launches / n_new, 3),
                           "greedy_launches": int(g0.launches), "llma_launches": int(tot),
                           "llma_steps": int(st.steps), "llma_ms_per_step": st.device_ms / st.steps}))
         return

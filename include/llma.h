@@ -117,8 +117,8 @@ typedef struct {
  * workspaces, among them, on the tensor-core path, 4 * (2 d_model + 2 n_heads*head_dim + d_ffn) bytes for each position of a
  * prompt pass (up to 2048 positions, 224 MB at the 7B widths; fewer positions, down to 128, where memory is short), and
  * a page-locked host block for tokens and references.  Engines whose decoding steps run whole in one launch also take 8 * (d_model +
- * 4 n_heads*head_dim + d_ffn + 2 * SMs) bytes for each row of a step, and launch kernel by kernel where memory is too short for that.  Supported: head_dim 64 or 128; d_model, n_heads*head_dim and d_ffn multiples
- * of 64; max_batch <= 256 and max_batch*(max_k+1) <= 256 rows per decoding step (the rows of a
+ * 4 n_heads*head_dim + d_ffn + 2 * SMs) bytes for each row of a step, and launch kernel by kernel where memory is too short for that
+ * or the stream has only some of the SMs.  Supported: head_dim 64 or 128; d_model, n_heads*head_dim and d_ffn multiples of 64; max_batch <= 256 and max_batch*(max_k+1) <= 256 rows per decoding step (the rows of a
  * step are packed, so a sequence without a copy takes one row).  Errors: NULL, CONFIG, CUDA.
  */
 int llma_create(const llma_config *cfg, const llma_weights *w, void *cuda_stream, llma_engine **out);
