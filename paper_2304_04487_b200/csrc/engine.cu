@@ -155,18 +155,29 @@ static cudaError_t init_whole_steps(llma_engine* e) {
     s.x = e->x; s.qkv = e->qkv; s.attn = (float*)e->attn; s.h = (float*)e->h; s.logits = e->cfg.keep_logits ? e->logits : nullptr;
     s.kcache = e->kcache; s.vcache = e->vcache; s.rope_cos = e->rope_cos; s.rope_sin = e->rope_sin;
     s.barrier = e->grid_barrier; s.dev_err = e->dev_err;
-    // A launch that does nothing: a stream that has only some of the SMs (a green context's) refuses one that needs them all
-    const int32_t off = kDevErrSteps, none = kDevErrNone;
-    SimtStep trial = s;
-    trial.tail.st = e->seq_state;
-    if ((r = cudaMemcpy(e->dev_err, &off, sizeof(off), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
-    if ((r = cudaDeviceSynchronize()) != cudaSuccess) return r;
-    const cudaError_t refused = launch_step_simt(e->stream, e->bf16, trial, e->simt_smem, e->num_sms);
-    if ((r = cudaStreamSynchronize(e->stream)) != cudaSuccess) return r;
-    if ((r = cudaMemcpy(e->dev_err, &none, sizeof(none), cudaMemcpyHostToDevice)) != cudaSuccess) return r;
-    cudaGetLastError();
-    e->step_simt = refused == cudaSuccess;
+    e->step_simt = true;
     return cudaSuccess;
+}
+
+// A launch that does nothing: a stream that has only some of the SMs (a green context's) refuses one that needs them all.  In its turn like
+// any other: a launch that waits for all SMs holds up the projections of other streams that wait for the rest of theirs.
+static cudaError_t try_whole_steps(llma_engine* e, bool* refused) {
+    const int32_t off = kDevErrSteps, none = kDevErrNone;
+    SimtStep trial = e->simt;
+    trial.tail.st = e->seq_state;
+    cudaError_t r = cudaMemcpy(e->dev_err, &off, sizeof(off), cudaMemcpyHostToDevice);
+    if (r == cudaSuccess) r = cudaDeviceSynchronize();
+    if (r != cudaSuccess) return r;
+    {
+        GateCall call(e->gate);
+        GateTurn turn(e->gate, kTurnSteps, e->num_sms);
+        if ((r = turn.error()) != cudaSuccess) return r;
+        *refused = launch_step_simt(e->stream, e->bf16, trial, e->simt_smem, e->num_sms) != cudaSuccess;
+        if ((r = turn.end()) != cudaSuccess) return r;
+        if ((r = cudaStreamSynchronize(e->stream)) != cudaSuccess) return r;
+    }
+    cudaGetLastError();
+    return cudaMemcpy(e->dev_err, &none, sizeof(none), cudaMemcpyHostToDevice);
 }
 
 extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* cuda_stream, llma_engine** out) {
@@ -418,6 +429,15 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     CREATE_TRY(cudaEventCreate(&e->ev0));
     CREATE_TRY(cudaEventCreate(&e->ev1));
     CREATE_TRY(gate_join(&e->gate, dev, e->stream, e->step_simt));
+    if (e->step_simt) {
+        bool refused = false;
+        CREATE_TRY(try_whole_steps(e, &refused));
+        if (refused) {
+            e->step_simt = false;
+            gate_quit(&e->gate);
+            CREATE_TRY(gate_join(&e->gate, dev, e->stream, false));
+        }
+    }
     CREATE_TRY(cudaDeviceSynchronize());
 #undef CREATE_TRY
     llma::gemm_count_engine(dev, 1);

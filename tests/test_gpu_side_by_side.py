@@ -59,14 +59,9 @@ def _product(noalloc):
     return work
 
 
-@pytest.mark.parametrize("whole,tiles", [("tiny-fp32", "mid-bf16"), ("small-bf16", "mid-bf16"), ("tiny-bf16", "llama7b-1layer")])
-def test_whole_steps_beside_other_engines(whole, tiles):
-    a, ya = _engine(whole, 4)
-    b, yb = _engine(whole, 4)
-    c, yc = _engine(tiles, 8)
-    jobs = [lambda: (_generate(a, ya, 4), _replay(a, ya, 4)), lambda: (_step(b, yb, 4), _generate(b, yb, 4)),
-            lambda: (_generate(c, yc, 8), _step(c, yc, 8), _replay(c, yc, 8)), _product(False), _product(True)]
-    failed, done, until = [], [0] * len(jobs), time.monotonic() + 1.0
+def _side_by_side(jobs, seconds):
+    """Every job again and again in a thread of its own, for some time."""
+    failed, done, until = [], [0] * len(jobs), time.monotonic() + seconds
 
     def loop(i):
         try:
@@ -82,8 +77,41 @@ def test_whole_steps_beside_other_engines(whole, tiles):
     for t in threads:
         t.join()
     assert not failed and min(done) > 0, (failed, done)
+
+
+@pytest.mark.parametrize("whole,tiles", [("tiny-fp32", "mid-bf16"), ("small-bf16", "mid-bf16"), ("tiny-bf16", "llama7b-1layer")])
+def test_whole_steps_beside_other_engines(whole, tiles):
+    a, ya = _engine(whole, 4)
+    b, yb = _engine(whole, 4)
+    c, yc = _engine(tiles, 8)
+    jobs = [lambda: (_generate(a, ya, 4), _replay(a, ya, 4)), lambda: (_step(b, yb, 4), _generate(b, yb, 4)),
+            lambda: (_generate(c, yc, 8), _step(c, yc, 8), _replay(c, yc, 8)), _product(False), _product(True)]
+    _side_by_side(jobs, 1.0)
     for e in (a, b, c):
         e.llma_destroy()
+
+
+def test_engines_come_and_go_beside_others():
+    """Engines of both kinds are made, used and destroyed while others decode: what a new engine launches takes turns from its first
+    launch on, the one that its creation makes included."""
+    import torch
+    from paper_2304_04487_b200 import Engine
+    old, y = _engine("mid-bf16", 8)
+    names = ("tiny-fp32", "mid-bf16", "tiny-bf16")
+    weights = {n: make_weights(SHAPES[n], seed=0) for n in names}
+    streams = {n: torch.cuda.Stream() for n in names}       # (streams of torch's pool come round again)
+    want = {}
+
+    def make():
+        for n in names:
+            eng = Engine(SHAPES[n], weights[n], max_seq=120, max_ref=16, max_k=2, stream=streams[n])
+            eng.llma_prefill(0, make_prompt(50, SHAPES[n].vocab, seed=9))
+            (toks,), _ = eng.llma_generate(20, 1, 0)
+            assert want.setdefault(n, toks) == toks
+            eng.llma_destroy()
+    make()
+    _side_by_side([make, lambda: (_generate(old, y, 8), _replay(old, y, 8)), _product(False)], 2.0)
+    old.llma_destroy()
 
 
 def test_stream_that_has_part_of_the_sms():
