@@ -1,11 +1,11 @@
 // Turns of kernels whose CTAs wait for one another (library-private).
 //
 // A whole-step launch (step_simt.cu) and a projection that adds up partial tiles (gemm_tcgen05.cu, gemm_wide.cu) need all of their CTAs on
-// the GPU before any of them can finish.  The GPU gives SMs that come free to CTAs of several streams in turn, so one kernel of each kind
-// can end up with some of the SMs each and wait for the others' until its waits run out: a whole-step engine beside a tensor-core engine
-// did, within milliseconds of starting both.  So launches of the two kinds from different streams take turns: whoever launches has its
-// stream wait for what calls under way on other streams have launched of the other kind.  (Projections of several streams go on side by
-// side, as do kernels without such waits.)  Only engines of one device concern each other, and only where one takes whole steps.
+// the GPU before any of them can finish.  Side by side on two streams, one of each kind can stop the other, with some of the SMs
+// each, until its waits run out: a whole-step engine beside a tensor-core engine did, within milliseconds of starting both.  So
+// launches of the two kinds from different streams take turns: whoever launches has its stream wait for what calls under way on other streams
+// have launched of the other kind.  (Projections of several streams go on side by side, as do kernels without such waits.)  Only
+// engines of one device concern each other, and only where one takes whole steps.
 //
 // Whole-step launches of several streams share the SMs: each takes as many CTAs as there are SMs for every call under way that takes
 // whole steps, down to a quarter (what a step gives does not depend on the number of CTAs), and waits for the oldest launches that hold

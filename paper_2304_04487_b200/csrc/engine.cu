@@ -116,16 +116,28 @@ static bool whole_steps_pay(const llma_engine* e, const SimtStep& s) {
            rows * (layer + head) <= 190000ll * (1100 - d.max_seq);
 }
 
+// A stream of a green context has some of the SMs only, where a launch that needs them all would never get its CTAs together.
+static bool has_every_sm(const llma_engine* e) {
+    auto entry = [](const char* name) -> void* {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        return cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess ? p : nullptr;
+    };
+    auto of_stream = reinterpret_cast<CUresult (*)(CUstream, CUgreenCtx*)>(entry("cuStreamGetGreenCtx"));
+    auto resource = reinterpret_cast<CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType)>(entry("cuGreenCtxGetDevResource"));
+    CUgreenCtx green = nullptr;
+    CUdevResource sms;
+    if (!of_stream || !resource || of_stream(e->stream, &green) != CUDA_SUCCESS || !green) return true;
+    return resource(green, &sms, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && (int)sms.sm.smCount >= e->num_sms;
+}
+
 // Whole decoding steps in one launch, where they are possible and pay
 static cudaError_t init_whole_steps(llma_engine* e) {
     const ModelDims& d = e->dims;
-    int coop = 0;
-    cudaError_t r = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, e->device);
-    if (r != cudaSuccess) return r;
     SimtStep& s = e->simt;
     bool fits = false;
-    if (!coop || !step_simt_shape(d, e->bf16, e->y_cap, e->num_sms, &s, &e->simt_smem) || !whole_steps_pay(e, s)) return cudaSuccess;
-    r = init_step_simt(e->bf16, d.head_dim, e->simt_smem, &fits);
+    if (!step_simt_shape(d, e->bf16, e->y_cap, e->num_sms, &s, &e->simt_smem) || !whole_steps_pay(e, s) || !has_every_sm(e)) return cudaSuccess;
+    cudaError_t r = init_step_simt(e->bf16, d.head_dim, e->simt_smem, &fits);
     if (r != cudaSuccess || !fits) return r;
     std::vector<SimtOp> ops;
     for (int l = 0; l < d.n_layers; ++l) {
@@ -157,27 +169,6 @@ static cudaError_t init_whole_steps(llma_engine* e) {
     s.barrier = e->grid_barrier; s.dev_err = e->dev_err;
     e->step_simt = true;
     return cudaSuccess;
-}
-
-// A launch that does nothing: a stream that has only some of the SMs (a green context's) refuses one that needs them all.  In its turn like
-// any other: a launch that waits for all SMs holds up the projections of other streams that wait for the rest of theirs.
-static cudaError_t try_whole_steps(llma_engine* e, bool* refused) {
-    const int32_t off = kDevErrSteps, none = kDevErrNone;
-    SimtStep trial = e->simt;
-    trial.tail.st = e->seq_state;
-    cudaError_t r = cudaMemcpy(e->dev_err, &off, sizeof(off), cudaMemcpyHostToDevice);
-    if (r == cudaSuccess) r = cudaDeviceSynchronize();
-    if (r != cudaSuccess) return r;
-    {
-        GateCall call(e->gate);
-        GateTurn turn(e->gate, kTurnSteps, e->num_sms);
-        if ((r = turn.error()) != cudaSuccess) return r;
-        *refused = launch_step_simt(e->stream, e->bf16, trial, e->simt_smem, e->num_sms) != cudaSuccess;
-        if ((r = turn.end()) != cudaSuccess) return r;
-        if ((r = cudaStreamSynchronize(e->stream)) != cudaSuccess) return r;
-    }
-    cudaGetLastError();
-    return cudaMemcpy(e->dev_err, &none, sizeof(none), cudaMemcpyHostToDevice);
 }
 
 extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* cuda_stream, llma_engine** out) {
@@ -429,15 +420,6 @@ extern "C" int llma_create(const llma_config* cfg, const llma_weights* w, void* 
     CREATE_TRY(cudaEventCreate(&e->ev0));
     CREATE_TRY(cudaEventCreate(&e->ev1));
     CREATE_TRY(gate_join(&e->gate, dev, e->stream, e->step_simt));
-    if (e->step_simt) {
-        bool refused = false;
-        CREATE_TRY(try_whole_steps(e, &refused));
-        if (refused) {
-            e->step_simt = false;
-            gate_quit(&e->gate);
-            CREATE_TRY(gate_join(&e->gate, dev, e->stream, false));
-        }
-    }
     CREATE_TRY(cudaDeviceSynchronize());
 #undef CREATE_TRY
     llma::gemm_count_engine(dev, 1);

@@ -79,7 +79,7 @@ struct llma_engine {
     int attn_tiles = 1;             // 128-position tiles per attention CTA in decoding steps (a function of the capacity only)
     float *attn_ws_o = nullptr, *attn_ws_ml = nullptr;
 
-    // whole steps in one cooperative launch (step_simt.cu): CUDA-core path, and narrow decoders of the tensor-core path
+    // whole steps in one launch (step_simt.cu): CUDA-core path, and narrow decoders of the tensor-core path
     bool step_simt = false;
     bool plain_acts = false;        // attn and h hold fp32 rows (of a whole step), whatever the path
     llma::SimtStep simt{};          // everything that does not change from launch to launch

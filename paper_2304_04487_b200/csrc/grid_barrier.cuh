@@ -1,4 +1,4 @@
-// A barrier over all CTAs of a cooperative launch, one word of global memory, by the scheme of the grid barrier in CUDA's cooperative
+// A barrier over all CTAs of a launch that are on the GPU together, one word of global memory, by the scheme of the grid barrier in CUDA's cooperative
 // groups, split into arrival and wait: CTA 0 adds 2^31 - (CTAs - 1), every other CTA 1, so the top bit flips when the last one has
 // arrived and the word is ready for the next round (and the next launch, of as many CTAs as it likes) as it is.
 //

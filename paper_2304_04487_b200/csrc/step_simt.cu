@@ -1,5 +1,5 @@
 // Whole decoding steps on the CUDA cores (decoders of the CUDA-core path and narrow bf16 decoders, where that pays: the rule and what it
-// measured are in engine.cu) in one cooperative launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
+// measured are in engine.cu) in one launch: embedding gather, layers, LM head, acceptance and the next plan, step after step.
 //
 // At the widths this path serves a step is a chain of short phases and costs their latency.  As launches of their own
 // (kernels_simt.cu, attention_simt.cu) a phase is released about 1 us after its predecessor has ended, fetches its rows, and runs
@@ -934,7 +934,9 @@ cudaError_t init_step_simt(bool bf16, int head_dim, size_t smem, bool* fits) {
 template <typename T, int HD>
 static cudaError_t launch_typed(cudaStream_t st, const SimtStep& s, size_t smem, int ctas) {
     void* args[] = {const_cast<SimtStep*>(&s)};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(step_simt_kernel<T, HD>), dim3(ctas), dim3(kThreads), args, smem, st);
+    // (Not a cooperative launch: while one waits for all of its SMs to come free at once, no other stream's CTAs start, and a kernel whose
+    // CTAs wait for one another then waits for good.  A launch of these CTAs one by one that does not get them together gives up.)
+    return cudaLaunchKernel(reinterpret_cast<const void*>(step_simt_kernel<T, HD>), dim3(ctas), dim3(kThreads), args, smem, st);
 }
 cudaError_t launch_step_simt(cudaStream_t st, bool bf16, const SimtStep& s, size_t smem, int ctas) {
     if (bf16) return s.dims.head_dim == 128 ? launch_typed<__nv_bfloat16, 128>(st, s, smem, ctas) : launch_typed<__nv_bfloat16, 64>(st, s, smem, ctas);
